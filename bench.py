@@ -385,7 +385,11 @@ def run_ours(args):
         return lp.pdhg_solve(TOL, ITER_CAP)
 
     def launches(res):
-        return 1 + int(res.launches)  # the cold reset plus what the solve issued
+        # the cold reset plus what the solve issued; a chunk of the resident form is one
+        # launch of its attempts and two of its check, and one chunk is queued ahead
+        if mixed.resident()[0]:
+            return 1 + 3 + 3 * (-(-int(res.iterations) // nchk) + 1)
+        return 1 + int(res.launches)
 
     for _ in range(args.warmup):
         step(mixed)

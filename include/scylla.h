@@ -156,7 +156,8 @@ typedef struct {
   double pobj, dobj;     /* primal/dual objective (with the objective offset) */
   double eta, omega;     /* step size and primal weight after the solve */
   double seconds;        /* device time of the solve (CUDA events) */
-  int64_t launches;      /* kernel launches issued, including ones that returned early */
+  int64_t launches;      /* kernel launches issued, including ones that returned early; an attempt of the
+                            resident form (scylla_resident) counts as the two launches it stands for */
   int32_t kernel_form;   /* form of the primal per-attempt kernel (scylla_params.prefetch's numbering: 4
                             32-row tiles, 1 32-row with prefetch, 2 wide tiles, 3 staged wide tiles); 0 for
                             the batched and fan-out solves */
@@ -290,6 +291,14 @@ int scylla_time_kernels(scylla_lp* lp, int32_t attempts, double* ms);
  * each kernel's form on its own.  Any output may be NULL. */
 int scylla_kernel_form(const scylla_lp* lp, int32_t* form, int32_t* form_dual, int32_t* rule_form,
                        double* tune_ms);
+
+/* Whether the handle's attempts run resident, all those between two checks in one
+ * launch: *scope = 0 no (two launches per attempt), 1 in one cluster of *blocks blocks,
+ * 2 in a cooperative grid of *blocks blocks.  Taken with use_graph = 1 and prefetch = 0
+ * for LPs that the L2-size rule gives 32-row tiles and whose tiles fit the blocks' shared
+ * memory; the results are those of the launched 32-row form bit for bit.  Either output
+ * may be NULL. */
+int scylla_resident(const scylla_lp* lp, int32_t* scope, int32_t* blocks);
 
 /* Diagonal scaling A~ = diag(R) A diag(C) found at create: host, R length m_total,
  * C length n_total. */

@@ -376,6 +376,20 @@ template <typename T>
 int persistent_blocks_per_sm();
 template <typename T>
 cudaError_t launch_persistent(const DevLP<T>& d, void* grid_bar, int grid, double wait_limit_s, cudaStream_t st);
+// the resident form of the per-attempt kernels (attempts.cuh): its launch for an LP
+// (false when it cannot run), and the launch of up to n_check attempts; bar:
+// kGridBarBytes
+struct ResidentPlan {
+  int scope;             // 0 none, 1 a cluster of blocks, 2 a grid of one block per SM
+  int blocks, threads;
+  int tpw;               // most tiles of a side per warp
+  int slots_t, slots_a;  // tile slots per block in shared memory, of the transpose and of A
+  size_t smem;           // dynamic shared memory per block
+};
+template <typename T>
+bool resident_plan(const DevLP<T>& d, ResidentPlan* out);
+template <typename T>
+cudaError_t launch_attempts(const DevLP<T>& d, const ResidentPlan& p, void* bar, cudaStream_t st);
 constexpr int kPersistentPartials = 24;  // doubles per block in DevLP::pp_part
 constexpr size_t kGridBarBytes = 16;
 template <typename T>

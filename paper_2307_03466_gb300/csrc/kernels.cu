@@ -1415,6 +1415,8 @@ __global__ void __launch_bounds__(kThreads) k_check_rows(DevLP<T> d) {
   }
 }
 
+#include "attempts.cuh"
+
 // ------------------------------------------------------ persistent solve kernel ---
 // The whole solve in one cooperative launch (all blocks co-resident): per attempt a
 // primal phase and a dual phase separated by grid barriers; after the dual barrier
@@ -3046,6 +3048,8 @@ int occupancy_grid(int side, int form, int work_tiles) {
   template cudaError_t launch_init_point<T>(const DevLP<T>&, cudaStream_t);                               \
   template int occupancy_grid<T>(int, int, int);                                                           \
   template int persistent_blocks_per_sm<T>();                                                             \
+  template bool resident_plan<T>(const DevLP<T>&, ResidentPlan*);                                         \
+  template cudaError_t launch_attempts<T>(const DevLP<T>&, const ResidentPlan&, void*, cudaStream_t);      \
   template cudaError_t launch_persistent<T>(const DevLP<T>&, void*, int, double, cudaStream_t);
 
 SCYLLA_INSTANTIATE(double)

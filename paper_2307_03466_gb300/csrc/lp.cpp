@@ -614,7 +614,7 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
     for (int k = 0; k < 2; ++k) lp->ATY[k] = ar.take<char>(vs * n);
     lp->XLR = ar.take<char>(vs * n);
     lp->YLR = ar.take<char>(vs * m);
-    lp->part_p = ar.take<double>(size_t(kNP) * std::max(cap_p, 1));
+    lp->part_p = ar.take<double>(2 * size_t(kNP) * std::max(cap_p, 1));  // the resident form's two buffers
     lp->part_d = ar.take<double>(size_t(kND) * std::max(cap_d, 1));
     lp->part_c1 = ar.take<double>(size_t(kNC1) * std::max(cap_c1, 1));
     lp->part_c2 = ar.take<double>(size_t(kNC2) * std::max(lp->grid_c2, 1));
@@ -768,6 +768,15 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
     CK(launch_init_point<double>(lp->d64, st));
   }
   CK(cudaStreamSynchronize(st));
+  // LPs that stay in L2 (the rule's 32-row plain form) run their attempts resident
+  // (attempts.cuh) and need no choice of a launched form
+  if (lp->p.prefetch == 0 && lp->form_rule == kFormPlain) {
+    ResidentPlan plan{};
+    if (mixed ? resident_plan<float>(lp->d32, &plan) : resident_plan<double>(lp->d64, &plan)) {
+      lp->tune = false;
+      if (lp->p.use_graph == 1) lp->resident = plan;
+    }
+  }
   if (lp->tune) {
     const int rc = mixed ? autotune_form<float>(lp) : autotune_form<double>(lp);
     if (rc != SCYLLA_OK) return rc;
@@ -1003,8 +1012,15 @@ static int build_chunk_graph(scylla_lp* lp, const DevLP<T>& d) {
   cudaStream_t st = lp->st;
   CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
-  for (int s = 0; s < lp->p.n_check && e == cudaSuccess; ++s) e = launch_slot<T>(d, st);
-  if (e == cudaSuccess) e = launch_check<T>(d, st);
+  if (lp->resident.scope) {
+    e = launch_attempts<T>(d, lp->resident, lp->grid_bar, st);
+    DevLP<T> dc = d;
+    dc.pdl = 0;  // its predecessor is not a launch that triggers its successor
+    if (e == cudaSuccess) e = launch_check<T>(dc, st);
+  } else {
+    for (int s = 0; s < lp->p.n_check && e == cudaSuccess; ++s) e = launch_slot<T>(d, st);
+    if (e == cudaSuccess) e = launch_check<T>(d, st);
+  }
   cudaGraph_t g = nullptr;
   const cudaError_t e2 = cudaStreamEndCapture(st, &g);
   if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -1068,11 +1084,15 @@ static int solve_impl(scylla_lp* lp, const DevLP<T>& d, double tol, int64_t iter
       launches += per_chunk;
       return e;
     };
+    // the check at the iteration limit ends the solve, so no chunk is queued ahead past it
+    const long long need = (iter_limit + nchk - 1) / nchk;
     CK(enqueue(0));
     for (long long c = 0; c < max_chunks; ++c) {
-      if (c + 1 < max_chunks) CK(enqueue(c + 1));
+      const bool ahead = c + 1 < need;
+      if (ahead) CK(enqueue(c + 1));
       CK(cudaEventSynchronize(lp->ev_chunk[c & 1]));
       if (lp->h_done[c & 1]) break;
+      if (!ahead && c + 1 < max_chunks) CK(enqueue(c + 1));
     }
   } else {
     for (long long ch = 0; ch < max_chunks; ++ch) {
@@ -1798,6 +1818,13 @@ extern "C" int scylla_kernel_form(const scylla_lp* lp, int32_t* form, int32_t* f
   if (rule_form) *rule_form = api_form(lp->form_rule);
   if (tune_ms)
     for (int q = 0; q < 6; ++q) tune_ms[q] = lp->tune_ms[q];
+  return SCYLLA_OK;
+}
+
+extern "C" int scylla_resident(const scylla_lp* lp, int32_t* scope, int32_t* blocks) {
+  if (!lp) FAIL(SCYLLA_ERR_INVALID_ARG, "null handle");
+  if (scope) *scope = lp->resident.scope;
+  if (blocks) *blocks = lp->resident.blocks;
   return SCYLLA_OK;
 }
 

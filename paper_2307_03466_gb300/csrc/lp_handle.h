@@ -62,6 +62,7 @@ struct scylla_lp {
   double* pp_part = nullptr;
   unsigned long long* p_hash = nullptr;
   void* grid_bar = nullptr;
+  scylla::ResidentPlan resident{};  // resident form of the per-attempt kernels (scope 0: launched ones)
   int p_grid = 0;  // persistent grid (0: that mode is unavailable)
   int form_p = 0, form_d = 0;  // forms of the primal / dual per-attempt kernels (kForm*)
   int form_rule = 0;           // the form the L2-size rule gives

@@ -119,6 +119,7 @@ _SIGS = {
     "scylla_reset_state": (C.c_int, [_P]),
     "scylla_time_kernels": (C.c_int, [_P, C.c_int32, _D]),
     "scylla_kernel_form": (C.c_int, [_P, C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int32), _D]),
+    "scylla_resident": (C.c_int, [_P, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
     "scylla_primal_residual_noalloc": (C.c_int, [C.c_int64, _P, _P, _P, _P, _P, _P, _P, _P]),
     "scylla_batch_create": (C.c_int, [C.c_int32, C.POINTER(Csr), C.POINTER(_D), C.POINTER(_D), C.POINTER(_D),
                                       C.POINTER(_D), C.POINTER(_D), C.POINTER(Params), _P, C.POINTER(_P)]),
@@ -434,6 +435,13 @@ class LP:
         ms = np.zeros(6)
         _check(lib().scylla_kernel_form(self.h, C.byref(f), C.byref(fd), C.byref(r), _dp(ms)))
         return (f.value, fd.value), r.value, ms
+
+    def resident(self):
+        """(scope, blocks) of the resident form of the attempts, (0, 0) when they are
+        launched one by one -- scylla_resident."""
+        sc, b = C.c_int32(), C.c_int32()
+        _check(lib().scylla_resident(self.h, C.byref(sc), C.byref(b)))
+        return sc.value, b.value
 
     def time_kernels(self, attempts: int):
         """Mean device ms of (primal, dual, check-cols, check-rows) launches."""
