@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 #include <type_traits>
 
@@ -24,6 +25,50 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+// Warp sums of P values per lane (P a power of two, at most 32), the additions of
+// warp_sum in the same association: at each of the first log2 P steps a lane passes on
+// one half of its values and keeps the sums of the other, so P values take P - 1 + log2
+// (32 / P) additions per lane, not 5 P (FP64 additions are what bounds the kernels that
+// sum ten values: a warp's one occupies its scheduler's FP64 pipe for about 64 cycles).
+// v[0] holds the sum of value warp_sums_index<P>() afterwards, on every lane.
+template <int P, typename A>
+__device__ __forceinline__ void warp_sums(A (&v)[P]) {
+  const int lane = threadIdx.x & 31;
+  int n = P;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (n > 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int i = 0; i < P / 2; ++i) {
+        if (i < n / 2) {
+          const A keep = up ? v[i + n / 2] : v[i], pass = up ? v[i] : v[i + n / 2];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, pass, o);
+        }
+      }
+      n /= 2;
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
+  }
+}
+template <int P>
+__device__ __forceinline__ int warp_sums_index() {
+  return (threadIdx.x & 31) / (32 / P);
+}
+// put(k, sum) on one lane for each k of N values, in pieces of 8, 4, 2 and 1
+template <int N, int K0 = 0, typename A, typename Put>
+__device__ __forceinline__ void warp_sums_put(const A* v, Put&& put) {
+  if constexpr (N > 0) {
+    constexpr int P = N >= 8 ? 8 : N >= 4 ? 4 : N >= 2 ? 2 : 1;
+    A t[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) t[i] = v[i];
+    warp_sums<P>(t);
+    if ((threadIdx.x & (32 / P - 1)) == 0) put(K0 + warp_sums_index<P>(), t[0]);
+    warp_sums_put<N - P, K0 + P>(v + P, put);
+  }
 }
 __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
 #pragma unroll
@@ -190,12 +235,8 @@ __device__ __forceinline__ unsigned long long round_hash(long long j, double v) 
 template <int N, typename A>
 __device__ __forceinline__ void block_store_partials(const A (&v)[N], A* __restrict__ part) {
   __shared__ A sh[kMaxWarps][N];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    const A t = warp_sum(v[k]);
-    if (lane == 0) sh[w][k] = t;
-  }
+  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  warp_sums_put<N>(v, [&](int k, A t) { sh[w][k] = t; });
   __syncthreads();
   if (threadIdx.x < N) {
     A s = A(0);
@@ -597,40 +638,40 @@ static __device__ void step_control(Control* c, double dx2, double dy2, double i
 // go to the control block.  The FP32-mixed mode needs only the FP32 table, from
 // powf; the FP64 mode computes one FP64 power per thread (each is a long serial
 // chain on this part) and rounds it for the FP32 copy.
+// the table by nt threads (this one is thread t of them); first receives attempt k + 1's
+// FP32 factors
 template <typename T>
-static __device__ void fill_step_factors(Control* c, double* fac, int n_check);
-
-template <>
-__device__ void fill_step_factors<float>(Control* c, double* fac, int n_check) {
-  const long long k = c->k;
-  const float er = float(c->exp_red), eg = float(c->exp_grow);
+__device__ __forceinline__ void fill_step_table(long long k, double exp_red, double exp_grow, double* fac, int n_check,
+                                                int t, int nt, float* first) {
   float* facf = reinterpret_cast<float*>(fac + 2 * n_check);
-  for (int i = threadIdx.x; i < n_check; i += blockDim.x) {
-    const float kk = float(k + 1 + i + 1);
-    const float fr = 1.0f - powf(kk, -er), fg = 1.0f + powf(kk, -eg);
-    facf[2 * i] = fr;
-    facf[2 * i + 1] = fg;
-    if (i == 0) {
-      c->fr_f = fr;
-      c->fg_f = fg;
+  if constexpr (std::is_same<T, float>::value) {
+    const float er = float(exp_red), eg = float(exp_grow);
+    for (int i = t; i < n_check; i += nt) {
+      const float kk = float(k + 1 + i + 1);
+      const float fr = 1.0f - powf(kk, -er), fg = 1.0f + powf(kk, -eg);
+      facf[2 * i] = fr;
+      facf[2 * i + 1] = fg;
+      if (i == 0) {
+        first[0] = fr;
+        first[1] = fg;
+      }
+    }
+  } else {
+    for (int q = t; q < 2 * n_check; q += nt) {
+      const double kk = double(k + 1 + (q >> 1) + 1);
+      const double v = (q & 1) ? 1.0 + pow(kk, -exp_grow) : 1.0 - pow(kk, -exp_red);
+      fac[q] = v;
+      facf[q] = float(v);
+      if (q < 2) first[q] = float(v);
     }
   }
-  if (threadIdx.x == 0) c->k_fac = k;
 }
-
-template <>
-__device__ void fill_step_factors<double>(Control* c, double* fac, int n_check) {
-  const long long k = c->k;
-  float* facf = reinterpret_cast<float*>(fac + 2 * n_check);
-  for (int q = threadIdx.x; q < 2 * n_check; q += blockDim.x) {
-    const double kk = double(k + 1 + (q >> 1) + 1);
-    const double v = (q & 1) ? 1.0 + pow(kk, -c->exp_grow) : 1.0 - pow(kk, -c->exp_red);
-    fac[q] = v;
-    facf[q] = float(v);
-    if (q == 0) c->fr_f = float(v);
-    if (q == 1) c->fg_f = float(v);
-  }
-  if (threadIdx.x == 0) c->k_fac = k;
+// by the whole block, attempt k + 1's factors and k straight into the control block
+template <typename T>
+__device__ __forceinline__ void fill_step_factors(Control* c, double* fac, int n_check) {
+  static_assert(sizeof(float) * 2 == 8 && offsetof(Control, fg_f) == offsetof(Control, fr_f) + 4, "factor pair");
+  fill_step_table<T>(c->k, c->exp_red, c->exp_grow, fac, n_check, int(threadIdx.x), int(blockDim.x), &c->fr_f);
+  if (threadIdx.x == 0) c->k_fac = c->k;
 }
 
 // ------------------------------------------------------------------ checks ---
@@ -782,8 +823,10 @@ static __device__ void check_control(Control* c, const double* r, double* trace,
   derive_steps(c);
 }
 
-// warp form: lanes 0 and 1 evaluate the two points side by side (their square roots
-// and divisions are long FP64 chains), lane 0 decides.  Called by a whole warp.
+// warp form: lanes 0 to 7 evaluate the two points (their square roots and divisions are
+// long FP64 chains: the three parts of the relative error and the weighted error of both
+// take one square root, one division and one more square root side by side), lane 0
+// decides.  Called by a whole warp.
 // The control block is worked on in a shared-memory copy that the warp loads and
 // stores with coalesced word accesses (the decision logic's many field accesses
 // are then shared-memory ones).
@@ -796,10 +839,37 @@ static __device__ void check_control_warp(Control* c, const double* r, double* t
   constexpr int kWords = int(sizeof(Control) / 4);
   for (int i = lane; i < kWords; i += 32) reinterpret_cast<int*>(&sc)[i] = reinterpret_cast<const int*>(c)[i];
   __syncwarp();
-  if (lane < 2) {
-    const Eval e = make_eval(&sc, r, lane);
-    se[lane] = e;
-    swk[lane] = weighted_kkt(e, sc.omega);
+  {
+    // lane 2 u + q: quantity u of point q, as make_eval and weighted_kkt form it
+    const int q = lane & 1, u = (lane >> 1) & 3;
+    const double* cs = r + 5 * q;
+    const double* rs = r + kNC1 + 4 * q;
+    const double pobj = cs[2] + sc.offset, dobj = (rs[2] + cs[3]) + sc.offset, om = sc.omega;
+    const double root = sqrt(u == 0 ? rs[1] : cs[1]);
+    const double num = u < 2 ? root : u == 2 ? fabs(pobj - dobj) : cs[0];
+    const double den = u == 0 ? 1.0 + sc.bnorm : u == 1 ? 1.0 + sc.cnorm
+                       : u == 2 ? 1.0 + fabs(pobj) + fabs(dobj) : om * om;
+    const double quo = num / den;
+    const double g = pobj - dobj;
+    const double wk = sqrt(om * om * rs[0] + quo + g * g);  // u = 3
+    const double eps_d = __shfl_down_sync(0xffffffffu, quo, 2), eps_g = __shfl_down_sync(0xffffffffu, quo, 4);
+    if (lane < 2) {
+      Eval e;
+      e.rd_s2 = cs[0];
+      e.rd2 = cs[1];
+      e.pobj = pobj;
+      e.dobj = dobj;
+      e.dx2 = cs[4];
+      e.rp_s2 = rs[0];
+      e.rp2 = rs[1];
+      e.dy2 = rs[3];
+      e.eps_p = quo;
+      e.eps_d = eps_d;
+      e.eps_g = eps_g;
+      e.rel = fmax(e.eps_p, fmax(e.eps_d, e.eps_g));
+      se[lane] = e;
+    }
+    if (lane == 6 || lane == 7) swk[q] = wk;
   }
   __syncwarp();
   if (lane == 0) {
@@ -818,7 +888,7 @@ struct AccOf {
 };
 
 // flags of a per-LP / per-objective slot
-constexpr int kSlotActive = 1, kSlotCopyLr = 2, kSlotCached = 4, kSlotAvg = 8, kSlotCheck = 16;
+constexpr int kSlotActive = 1, kSlotCopyLr = 2, kSlotCached = 4, kSlotAvg = 8, kSlotCheck = 16, kSlotHash = 32;
 
 template <typename T>
 __device__ __forceinline__ void write_slot(BatchSlot<T>* s, const Control* c) {
@@ -838,6 +908,7 @@ __device__ __forceinline__ void write_slot(BatchSlot<T>* s, const Control* c) {
   if (c->copy_lr) f |= kSlotCopyLr;
   if (c->aty_valid) f |= kSlotCached;
   if (c->avg_w > 0.0) f |= kSlotAvg;
+  if (c->stall_checks > 0) f |= kSlotHash;
   v.flags = f;
   *s = v;
 }

@@ -167,7 +167,7 @@ struct DevBatch {
   unsigned int* lp_cnt;       // per LP: tiles of A done in this attempt's dual step (the last one decides)
   long long* kglob;           // attempts made by the LPs still running
   double exp_red, exp_grow;
-  int grid_p, grid_d, grid_c1, grid_c2, grid_ctl;
+  int grid_p, grid_d, grid_c1, grid_c2;
   int async_p, async_d;       // FP32: the primal / dual attempt kernel stages each warp's next tile by
                               // asynchronous copies
   int grid_pa, grid_da;       // their grids

@@ -1224,6 +1224,7 @@ struct CheckColsEpi {
   const unsigned char* int_mask;
   T w, w1;
   bool do_avg;
+  bool hash_on;  // the rounded point's hash only feeds the stall test
   double acc[kNC1];
   unsigned long long h;
   __device__ __forceinline__ Pre load(int) const { return Pre{}; }
@@ -1265,7 +1266,7 @@ struct CheckColsEpi {
       const double dd = xs[q] - xl;
       acc[5 * q + 4] += dd * dd;
     }
-    if (int_mask[j]) h += round_hash(j, xs[0] * Cj);
+    if (hash_on && int_mask[j]) h += round_hash(j, xs[0] * Cj);
   }
 };
 
@@ -1274,7 +1275,7 @@ struct CheckColsEpi {
 // rounding hash; block partials to part, hash into *hash
 template <typename T, bool Coh, int QP = 0>
 __device__ __forceinline__ void check_cols_phase(const DevLP<T>& d, const SlotView<T>& v, double* sm, double* part,
-                                                 unsigned long long* hash) {
+                                                 unsigned long long* hash, bool hash_on) {
   const T w = v.w, w1 = v.w1;
   const bool do_avg = v.do_avg;
   const T* __restrict__ yc = d.Y[v.cur];
@@ -1295,6 +1296,7 @@ __device__ __forceinline__ void check_cols_phase(const DevLP<T>& d, const SlotVi
   epi.w = w;
   epi.w1 = w1;
   epi.do_avg = do_avg;
+  epi.hash_on = hash_on;
 #pragma unroll
   for (int k = 0; k < kNC1; ++k) epi.acc[k] = 0.0;
   epi.h = 0ULL;
@@ -1386,7 +1388,7 @@ __global__ void __launch_bounds__(kThreads) k_check_cols(DevLP<T> d) {
   pdl_enter();
   if (ctl->done) return;
   __shared__ double sm[2 * kWarpsPerBlock * kSmemPerWarp];
-  check_cols_phase<T, false, QP>(d, make_view<T>(ctl), sm, d.part_c1, &ctl->hash_accum);
+  check_cols_phase<T, false, QP>(d, make_view<T>(ctl), sm, d.part_c1, &ctl->hash_accum, ctl->stall_checks > 0);
 }
 
 template <typename T>
@@ -1406,12 +1408,24 @@ __global__ void __launch_bounds__(kThreads) k_check_rows(DevLP<T> d) {
   static_assert(kNC2 * (kThreads - 32) <= 2 * kWarpsPerBlock * kSmemPerWarp, "reduction scratch");
   if (threadIdx.x < kNC1) red[threadIdx.x] = __ldcg(d.red_c1 + threadIdx.x);
   reduce_one<kNC2>(d.part_c2, d.grid_c2, sm, red + kNC1);
-  fill_step_factors<T>(ctl, d.step_fac, d.n_check);
+  // the decision (warp 0) beside the factor table (the other warps); attempt k + 1's
+  // factors go to the control block once the decision has written it back
+  __shared__ float first[2];
+  const long long k = ctl->k;
   if (threadIdx.x < 32) {
     if (threadIdx.x == 0 && std::is_same<T, float>::value) sync_step_state(ctl);
     __syncwarp();
     check_control_warp(ctl, red, d.trace_checks, d.trace_cap);
     if (threadIdx.x == 0) ctl->cnt_c2 = 0;
+  } else {
+    fill_step_table<T>(k, ctl->exp_red, ctl->exp_grow, d.step_fac, d.n_check, int(threadIdx.x) - 32,
+                       int(blockDim.x) - 32, first);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ctl->fr_f = first[0];
+    ctl->fg_f = first[1];
+    ctl->k_fac = k;
   }
 }
 
@@ -1501,7 +1515,7 @@ __global__ void __launch_bounds__(kPThreads, 1) k_solve_persistent(DevLP<T> d, G
   while (ok) {
     if (do_check) {
       const SlotView<T> v = make_view<T>(&sc);
-      check_cols_phase<T, true, 2>(d, v, psm, part_c1, &hash[hslot]);
+      check_cols_phase<T, true, 2>(d, v, psm, part_c1, &hash[hslot], sc.stall_checks > 0);
       ok = grid_sync(bar, limit_ns);
       if (!ok) break;
       check_rows_phase<T, true>(d, v, psm, part_c2);
@@ -1788,18 +1802,32 @@ __global__ void k_cnorm_cols(DevObjective o, double offset_base) {
 
 // One warp tile of the batched kernels (a multi-row tile or one long row): the
 // products into the warp's skewed shared buffer, then each lane sums its row in CSR
-// order and hands it to the epilogue.
-template <int NV, typename Acc, typename V, typename Gather, typename Epi>
+// order and hands it to the epilogue.  FMA: the checks of FP32 iterates (gat gives the
+// FP32 entries): values and entries into the buffer, and every row sum a chain of FP64
+// fused multiply-adds with exactly converted entries, as in spmv_tiles_fma (one FP64
+// instruction per nonzero and vector, not a conversion, a product and a sum).
+template <int NV, bool FMA, typename Acc, typename V, typename Gather, typename Epi>
 __device__ __forceinline__ void batch_tile_at(int2 ta, int2 tb, const int* __restrict__ rowptr,
                                               const int* __restrict__ cols, const V* __restrict__ vals, Gather& gat,
                                               Epi& epi, Acc* __restrict__ sm) {
+  float* __restrict__ sg = reinterpret_cast<float*>(sm + kSmemPerWarp);  // FMA: the entries
   const int lane = threadIdx.x & 31;
   const int r0 = ta.x, r1 = tb.x, p0 = ta.y, p1 = tb.y;
   const int base = p0 & ~(kVec - 1);
   if (r1 - r0 == 1 && p1 - p0 > kTileNnz) {
     const typename Epi::Pre pre = epi.load(r0);
     Acc s[NV];
-    long_row_sum<NV, false>(p0, p1, cols, vals, gat, s);
+    if constexpr (FMA) {
+      auto wide = [&](int i, Acc(&g)[NV]) {
+        float f[NV];
+        gat(i, f);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) g[k] = to_f64(f[k]);
+      };
+      long_row_sum<NV, false>(p0, p1, cols, vals, wide, s);
+    } else {
+      long_row_sum<NV, false>(p0, p1, cols, vals, gat, s);
+    }
     if (lane == 0) epi.finish(r0, s, pre);
   } else {
     const bool mine = lane < r1 - r0;
@@ -1828,11 +1856,19 @@ __device__ __forceinline__ void batch_tile_at(int2 ta, int2 tb, const int* __res
       for (int e = 0; e < 4; ++e) {
         const int q = p + e;
         if (q >= p0 && q < p1) {
-          Acc g[NV];
-          gat(c[it][e], g);
           const int o = skew(q - p0);
+          if constexpr (FMA) {
+            float g[NV];
+            gat(c[it][e], g);
+            sm[o] = v[it][e];
 #pragma unroll
-          for (int k = 0; k < NV; ++k) sm[k * kSmemPerWarp + o] = Acc(v[it][e]) * g[k];
+            for (int k = 0; k < NV; ++k) sg[k * kSmemPerWarp + o] = g[k];
+          } else {
+            Acc g[NV];
+            gat(c[it][e], g);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) sm[k * kSmemPerWarp + o] = Acc(v[it][e]) * g[k];
+          }
         }
       }
     }
@@ -1843,8 +1879,14 @@ __device__ __forceinline__ void batch_tile_at(int2 ta, int2 tb, const int* __res
       for (int k = 0; k < NV; ++k) s[k] = Acc(0);
       for (int q = q0; q < q1; ++q) {
         const int o = skew(q);
+        if constexpr (FMA) {
+          const Acc a = sm[o];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) s[k] += sm[k * kSmemPerWarp + o];
+          for (int k = 0; k < NV; ++k) s[k] = fma_t<Acc>(a, to_f64(sg[k * kSmemPerWarp + o]), s[k]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < NV; ++k) s[k] += sm[k * kSmemPerWarp + o];
+        }
       }
       epi.finish(row, s, pre);
     }
@@ -1853,11 +1895,11 @@ __device__ __forceinline__ void batch_tile_at(int2 ta, int2 tb, const int* __res
 }
 
 // tile t of a batch: its bounds, then batch_tile_at
-template <int NV, typename Acc, typename V, typename Gather, typename Epi>
+template <int NV, bool FMA, typename Acc, typename V, typename Gather, typename Epi>
 __device__ __forceinline__ void batch_tile(int t, const int2* __restrict__ tiles, const int* __restrict__ rowptr,
                                            const int* __restrict__ cols, const V* __restrict__ vals, Gather& gat,
                                            Epi& epi, Acc* __restrict__ sm) {
-  batch_tile_at<NV, Acc, V>(__ldg(tiles + t), __ldg(tiles + t + 1), rowptr, cols, vals, gat, epi, sm);
+  batch_tile_at<NV, FMA, Acc, V>(__ldg(tiles + t), __ldg(tiles + t + 1), rowptr, cols, vals, gat, epi, sm);
 }
 
 // warp-tile loop of the batched kernels over a static deal of the tiles:
@@ -1865,7 +1907,7 @@ __device__ __forceinline__ void batch_tile(int t, const int2* __restrict__ tiles
 // takes part, end(t) flushes the tile's sums.  The LP index and the bounds of the
 // warp's next tile are loaded together, one tile ahead, so that neither waits on
 // the other nor on the current tile's work.
-template <int NV, typename Acc, typename V, typename Gather, typename Epi>
+template <int NV, bool FMA, typename Acc, typename V, typename Gather, typename Epi>
 __device__ __forceinline__ void spmv_tiles_batch(const int2* __restrict__ tiles, const int* __restrict__ tile_lp,
                                                  int ntiles, const int* __restrict__ rowptr,
                                                  const int* __restrict__ cols, const V* __restrict__ vals,
@@ -1886,7 +1928,7 @@ __device__ __forceinline__ void spmv_tiles_batch(const int2* __restrict__ tiles,
     const int2 ta = ta_n, tb = tb_n;
     ahead(t + wt.step);
     if (!epi.begin(lp, t)) continue;
-    batch_tile_at<NV, Acc, V>(ta, tb, rowptr, cols, vals, gat, epi, sm);
+    batch_tile_at<NV, FMA, Acc, V>(ta, tb, rowptr, cols, vals, gat, epi, sm);
     epi.end(t);
   }
 }
@@ -2106,7 +2148,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_bprimal(DevBa
   epi.qq = nullptr;  // the batched solve takes LPs only
   epi.acc = 0;
   auto gat = [&](int i, T(&g)[1]) { g[0] = epi.cached ? T(0) : __ldg(epi.ysrc + i); };
-  spmv_tiles_batch<1, T, T>(d.t_tiles, B.t_tile_lp, d.t_ntiles, d.t_rowptr, d.t_cols, d.t_vals, gat, epi,
+  spmv_tiles_batch<1, false, T, T>(d.t_tiles, B.t_tile_lp, d.t_ntiles, d.t_rowptr, d.t_cols, d.t_vals, gat, epi,
                             sm + (threadIdx.x >> 5) * kSmemPerWarp);
 }
 
@@ -2246,14 +2288,54 @@ struct BDualEpi : DualEpi<T, Coh> {
   }
 };
 
-// one warp per LP: its tiles' sums in a fixed order, then the step decision (the
-// launch-per-phase path)
+// One lane's chain of per-tile values part[t * stride + off], t = beg, beg + step, ... <
+// end, added in that order; eight loads in flight.
+__device__ __forceinline__ double lp_chain_sum(const double* part, int stride, int off, int beg, int end, int step) {
+  double v = 0.0;
+  for (int t = beg; t < end; t += 8 * step) {
+    double x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = t + u * step < end ? __ldcg(part + size_t(t + u * step) * stride + off) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (t + u * step < end) v += x[u];
+  }
+  return v;
+}
+
+// A block per LP: its tiles' sums in lp_tile_sum's order, then the step decision (the
+// launch-per-phase path).  Warp 4 k + u takes the fourth u of sum k's running sums, so
+// the largest LP's chain is a twelfth of one warp's work and its loads come eight at a
+// time (64 LPs of up to 50k rows: 29 -> 9 us per attempt); the control block is decided on
+// in shared memory.
+constexpr int kBStepThreads = 12 * 32;
 template <typename T>
-__global__ void k_bstep_control(DevBatch<T> B) {
-  const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (b >= B.nlp) return;
+__global__ void __launch_bounds__(kBStepThreads) k_bstep_control(DevBatch<T> B) {
+  const int b = blockIdx.x;
   if (!(B.slot[b].flags & kSlotActive)) return;
-  lp_step_decision<T>(&B, b, nullptr);
+  __shared__ Control sc;
+  __shared__ double sh[12][32];
+  __shared__ double red[3];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, k = w >> 2, u = w & 3;
+  if (w == 11) ctl_in(&sc, B.ctl + b);
+  {
+    const int beg = __ldg((k == 0 ? B.t_tile_beg : B.a_tile_beg) + b);
+    const int end = __ldg((k == 0 ? B.t_tile_beg : B.a_tile_beg) + b + 1);
+    sh[w][lane] = lp_chain_sum(k == 0 ? B.tp_p : B.tp_d, k == 0 ? 1 : 2, k == 2 ? 1 : 0, beg + lane + 32 * u, end, 128);
+  }
+  __syncthreads();
+  if (w < 3) {
+    const double v = warp_sum((sh[4 * w][lane] + sh[4 * w + 1][lane]) + (sh[4 * w + 2][lane] + sh[4 * w + 3][lane]));
+    if (lane == 0) red[w] = v;
+  }
+  __syncthreads();
+  if (w == 0) {
+    if (lane == 0) {
+      bq_decide<T>(&sc, red[0], red[1], red[2], B.d.step_fac, B.d.n_check, &B.slot[b], B.n_done);
+      B.lp_cnt[b] = 0u;
+    }
+    ctl_out(B.ctl + b, &sc);
+  }
 }
 
 template <typename T>
@@ -2269,7 +2351,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_bdual(DevBatc
   epi.acc0 = 0;
   epi.acc1 = 0;
   auto gat = [&](int j, T(&g)[1]) { g[0] = __ldg(epi.xsrc + j); };
-  spmv_tiles_batch<1, T, T>(d.a_tiles, B.a_tile_lp, d.a_ntiles, d.a_rowptr, d.a_cols, d.a_vals, gat, epi,
+  spmv_tiles_batch<1, false, T, T>(d.a_tiles, B.a_tile_lp, d.a_ntiles, d.a_rowptr, d.a_cols, d.a_vals, gat, epi,
                             sm + (threadIdx.x >> 5) * kSmemPerWarp);
 }
 
@@ -2336,15 +2418,14 @@ struct BCheckColsEpi : CheckColsEpi<T, 0, Coh> {
     ycur = d.Y[s.cur];
     yavg = d.Y[s.avg];
     lp = b;
+    this->hash_on = (s.flags & kSlotHash) != 0;
     return true;
   }
   __device__ __forceinline__ void end(int t) {
+    warp_sums_put<kNC1>(this->acc, [&](int i, double a) { B->tp_c1[kNC1 * t + i] = a; });
 #pragma unroll
-    for (int k = 0; k < kNC1; ++k) {
-      const double a = warp_sum(this->acc[k]);
-      if ((threadIdx.x & 31) == 0) B->tp_c1[kNC1 * t + k] = a;
-      this->acc[k] = 0.0;
-    }
+    for (int k = 0; k < kNC1; ++k) this->acc[k] = 0.0;
+    if (!this->hash_on) return;
     const unsigned long long h = warp_sum_u64(this->h);
     if ((threadIdx.x & 31) == 0 && h != 0ULL) atomicAdd(&B->ctl[lp].hash_accum, h);
     this->h = 0ULL;
@@ -2368,14 +2449,14 @@ __global__ void __launch_bounds__(kThreads) k_bcheck_cols(DevBatch<T> B) {
 #pragma unroll
   for (int k = 0; k < kNC1; ++k) epi.acc[k] = 0.0;
   epi.h = 0ULL;
-  auto gat = [&](int i, double(&g)[2]) {
+  auto gat = [&](int i, T(&g)[2]) {
     const T y = epi.ycur[i];
     T av = epi.yavg[i];
     if (epi.bavg) av = blend(av, y, epi.bw1, epi.bw);
-    g[0] = double(y);
-    g[1] = double(av);
+    g[0] = y;
+    g[1] = av;
   };
-  spmv_tiles_batch<2, double, double>(d.t_tiles, B.t_tile_lp, d.t_ntiles, d.t_rowptr, d.t_cols, d.t_vals64, gat,
+  spmv_tiles_batch<2, sizeof(T) == 4, double, double>(d.t_tiles, B.t_tile_lp, d.t_ntiles, d.t_rowptr, d.t_cols, d.t_vals64, gat,
                                       epi, sm + (threadIdx.x >> 5) * 2 * kSmemPerWarp);
 }
 
@@ -2400,12 +2481,9 @@ struct BCheckRowsEpi : CheckRowsEpi<T, Coh> {
     return true;
   }
   __device__ __forceinline__ void end(int t) {
+    warp_sums_put<kNC2>(this->acc, [&](int i, double a) { B->tp_c2[kNC2 * t + i] = a; });
 #pragma unroll
-    for (int k = 0; k < kNC2; ++k) {
-      const double a = warp_sum(this->acc[k]);
-      if ((threadIdx.x & 31) == 0) B->tp_c2[kNC2 * t + k] = a;
-      this->acc[k] = 0.0;
-    }
+    for (int k = 0; k < kNC2; ++k) this->acc[k] = 0.0;
   }
 };
 
@@ -2421,46 +2499,47 @@ __global__ void __launch_bounds__(kThreads) k_bcheck_rows(DevBatch<T> B) {
   epi.hi64 = d.hi64;
 #pragma unroll
   for (int k = 0; k < kNC2; ++k) epi.acc[k] = 0.0;
-  auto gat = [&](int j, double(&g)[2]) {
-    g[0] = double(epi.xcur[j]);
-    g[1] = double(epi.xavg[j]);
+  auto gat = [&](int j, T(&g)[2]) {
+    g[0] = epi.xcur[j];
+    g[1] = epi.xavg[j];
   };
-  spmv_tiles_batch<2, double, double>(d.a_tiles, B.a_tile_lp, d.a_ntiles, d.a_rowptr, d.a_cols, d.a_vals64, gat,
+  spmv_tiles_batch<2, sizeof(T) == 4, double, double>(d.a_tiles, B.a_tile_lp, d.a_ntiles, d.a_rowptr, d.a_cols, d.a_vals64, gat,
                                       epi, sm + (threadIdx.x >> 5) * 2 * kSmemPerWarp);
 }
 
-// one warp per LP: its check sums in a fixed order, then termination / stalling /
-// restart (check_control); block 0 also refills the shared step-size factor table
-// for the next n_check attempts (every LP still running is at the same attempt)
+// A block per LP: its check sums in a fixed order (a warp per sum, a lane's tiles 32
+// apart), then termination / stalling / restart; one more block refills the shared
+// step-size factor table for the next n_check attempts (every LP still running is at the
+// same attempt)
+constexpr int kBCheckThreads = (kNC1 + kNC2) * 32;
 template <typename T>
-__global__ void k_bcheck_control(DevBatch<T> B) {
-  if (blockIdx.x == 0) {
+__global__ void __launch_bounds__(kBCheckThreads) k_bcheck_control(DevBatch<T> B) {
+  const int b = blockIdx.x;
+  if (b == B.nlp) {
     const long long k = *B.kglob;
-    for (int i = threadIdx.x; i < B.d.n_check; i += blockDim.x) {
-      const double kk = double(k + 1 + i + 1);
-      B.d.step_fac[2 * i] = 1.0 - pow(kk, -B.exp_red);
-      B.d.step_fac[2 * i + 1] = 1.0 + pow(kk, -B.exp_grow);
+    for (int q = threadIdx.x; q < 2 * B.d.n_check; q += blockDim.x) {
+      const double kk = double(k + 1 + (q >> 1) + 1);
+      B.d.step_fac[q] = (q & 1) ? 1.0 + pow(kk, -B.exp_grow) : 1.0 - pow(kk, -B.exp_red);
     }
+    return;
   }
-  const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (b >= B.nlp) return;
   if (!(B.slot[b].flags & kSlotCheck)) return;
-  double r[kNC1 + kNC2];
-#pragma unroll
-  for (int k = 0; k < kNC1 + kNC2; ++k) r[k] = 0.0;
-  for (int t = B.t_tile_beg[b] + lane; t < B.t_tile_beg[b + 1]; t += 32)
-#pragma unroll
-    for (int k = 0; k < kNC1; ++k) r[k] += B.tp_c1[kNC1 * t + k];
-  for (int t = B.a_tile_beg[b] + lane; t < B.a_tile_beg[b + 1]; t += 32)
-#pragma unroll
-    for (int k = 0; k < kNC2; ++k) r[kNC1 + k] += B.tp_c2[kNC2 * t + k];
-#pragma unroll
-  for (int k = 0; k < kNC1 + kNC2; ++k) r[k] = warp_sum(r[k]);
+  __shared__ double red[kNC1 + kNC2];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  {
+    const bool col = w < kNC1;
+    const int beg = __ldg((col ? B.t_tile_beg : B.a_tile_beg) + b), end = __ldg((col ? B.t_tile_beg : B.a_tile_beg) + b + 1);
+    const double v = warp_sum(lp_chain_sum(col ? B.tp_c1 : B.tp_c2, col ? kNC1 : kNC2, col ? w : w - kNC1, beg + lane,
+                                           end, 32));
+    if (lane == 0) red[w] = v;
+  }
+  __syncthreads();
+  if (w != 0) return;
+  Control* c = &B.ctl[b];
+  if (lane == 0) c->k_fac = *B.kglob;
+  __syncwarp();
+  check_control_warp(c, red, nullptr, 0);
   if (lane == 0) {
-    Control* c = &B.ctl[b];
-    c->k_fac = *B.kglob;
-    check_control(c, r, nullptr, 0);
     if (c->done) atomicAdd(B.n_done, 1);
     write_slot(&B.slot[b], c);
   }
@@ -2535,7 +2614,7 @@ constexpr int kQChunk = 4;          // tiles a warp takes from a queue at once
 // contiguous share of the first three quarters of the list (no atomics), then the
 // warps take the last quarter kQChunk tiles at a time from the shared counter, which
 // evens out the finishing times whatever the tiles' costs.
-template <int NV, typename Acc, typename V, typename Gather, typename Epi>
+template <int NV, bool FMA, typename Acc, typename V, typename Gather, typename Epi>
 __device__ __forceinline__ void queue_tiles(const int* list, int count, unsigned int* ctr, const int2* tiles,
                                             const int* tile_lp, const int* rowptr, const int* cols, const V* vals,
                                             Gather& gat, Epi& epi, Acc* sm) {
@@ -2544,7 +2623,7 @@ __device__ __forceinline__ void queue_tiles(const int* list, int count, unsigned
   auto one = [&](int v) {
     const int t = __ldcg(list + v);
     if (!epi.begin(__ldg(tile_lp + t), t)) return;
-    batch_tile<NV, Acc, V>(t, tiles, rowptr, cols, vals, gat, epi, sm);
+    batch_tile<NV, FMA, Acc, V>(t, tiles, rowptr, cols, vals, gat, epi, sm);
     epi.end(t);
   };
   const int per = int((3LL * count) / (4LL * nw));
@@ -2572,7 +2651,7 @@ __device__ __forceinline__ void bq_primal(const DevBatch<T>& B, int count, T* sm
   epi.qq = nullptr;
   epi.acc = 0;
   auto gat = [&](int i, T(&g)[1]) { g[0] = epi.cached ? T(0) : __ldcg(epi.ysrc + i); };
-  queue_tiles<1, T, T>(B.q_t, count, B.q_ctr + 0, d.t_tiles, B.t_tile_lp, d.t_rowptr, d.t_cols, d.t_vals, gat, epi,
+  queue_tiles<1, false, T, T>(B.q_t, count, B.q_ctr + 0, d.t_tiles, B.t_tile_lp, d.t_rowptr, d.t_cols, d.t_vals, gat, epi,
                        sm);
 }
 
@@ -2588,7 +2667,7 @@ __device__ __forceinline__ void bq_dual(const DevBatch<T>& B, int count, T* sm, 
   epi.acc0 = 0;
   epi.acc1 = 0;
   auto gat = [&](int j, T(&g)[1]) { g[0] = __ldcg(epi.xsrc + j); };
-  queue_tiles<1, T, T>(B.q_a, count, B.q_ctr + 1, d.a_tiles, B.a_tile_lp, d.a_rowptr, d.a_cols, d.a_vals, gat, epi,
+  queue_tiles<1, false, T, T>(B.q_a, count, B.q_ctr + 1, d.a_tiles, B.a_tile_lp, d.a_rowptr, d.a_cols, d.a_vals, gat, epi,
                        sm);
 }
 
@@ -2608,14 +2687,14 @@ __device__ __forceinline__ void bq_check_cols(const DevBatch<T>& B, int count, d
 #pragma unroll
   for (int k = 0; k < kNC1; ++k) epi.acc[k] = 0.0;
   epi.h = 0ULL;
-  auto gat = [&](int i, double(&g)[2]) {
+  auto gat = [&](int i, T(&g)[2]) {
     const T y = __ldcg(epi.ycur + i);
     T av = __ldcg(epi.yavg + i);
     if (epi.bavg) av = blend(av, y, epi.bw1, epi.bw);
-    g[0] = double(y);
-    g[1] = double(av);
+    g[0] = y;
+    g[1] = av;
   };
-  queue_tiles<2, double, double>(B.q_t, count, B.q_ctr + 2, d.t_tiles, B.t_tile_lp, d.t_rowptr, d.t_cols, d.t_vals64,
+  queue_tiles<2, sizeof(T) == 4, double, double>(B.q_t, count, B.q_ctr + 2, d.t_tiles, B.t_tile_lp, d.t_rowptr, d.t_cols, d.t_vals64,
                                  gat, epi, sm);
 }
 
@@ -2630,11 +2709,11 @@ __device__ __forceinline__ void bq_check_rows(const DevBatch<T>& B, int count, d
   epi.hi64 = d.hi64;
 #pragma unroll
   for (int k = 0; k < kNC2; ++k) epi.acc[k] = 0.0;
-  auto gat = [&](int j, double(&g)[2]) {
-    g[0] = double(__ldcg(epi.xcur + j));
-    g[1] = double(__ldcg(epi.xavg + j));
+  auto gat = [&](int j, T(&g)[2]) {
+    g[0] = __ldcg(epi.xcur + j);
+    g[1] = __ldcg(epi.xavg + j);
   };
-  queue_tiles<2, double, double>(B.q_a, count, B.q_ctr + 3, d.a_tiles, B.a_tile_lp, d.a_rowptr, d.a_cols, d.a_vals64,
+  queue_tiles<2, sizeof(T) == 4, double, double>(B.q_a, count, B.q_ctr + 3, d.a_tiles, B.a_tile_lp, d.a_rowptr, d.a_cols, d.a_vals64,
                                  gat, epi, sm);
 }
 
@@ -3079,14 +3158,14 @@ static void batch_attempt_kernels(const DevBatch<double>& B, cudaStream_t st, in
 template <typename T>
 cudaError_t launch_batch_slot(const DevBatch<T>& B, cudaStream_t st) {
   batch_attempt_kernels(B, st, -1);
-  k_bstep_control<T><<<B.grid_ctl, kThreads, 0, st>>>(B);
+  k_bstep_control<T><<<B.nlp, kBStepThreads, 0, st>>>(B);
   return cudaGetLastError();
 }
 // one kernel of an attempt on its own (measurement): 0 primal, 1 dual, 2 step control
 template <typename T>
 cudaError_t launch_batch_part(const DevBatch<T>& B, int part, cudaStream_t st) {
   if (part == 0 || part == 1) batch_attempt_kernels(B, st, part);
-  else k_bstep_control<T><<<B.grid_ctl, kThreads, 0, st>>>(B);
+  else k_bstep_control<T><<<B.nlp, kBStepThreads, 0, st>>>(B);
   return cudaGetLastError();
 }
 
@@ -3094,7 +3173,7 @@ template <typename T>
 cudaError_t launch_batch_check(const DevBatch<T>& B, cudaStream_t st) {
   k_bcheck_cols<T><<<B.grid_c1, kThreads, 0, st>>>(B);
   k_bcheck_rows<T><<<B.grid_c2, kThreads, 0, st>>>(B);
-  k_bcheck_control<T><<<B.grid_ctl, kThreads, 0, st>>>(B);
+  k_bcheck_control<T><<<B.nlp + 1, kBCheckThreads, 0, st>>>(B);
   return cudaGetLastError();
 }
 template <typename T>
@@ -3166,8 +3245,6 @@ void batch_grids(DevBatch<T>& B) {
   }
   B.grid_c1 = grid((const void*)k_bcheck_cols<T>, B.d.t_ntiles, 0);
   B.grid_c2 = grid((const void*)k_bcheck_rows<T>, B.d.a_ntiles, 0);
-  B.grid_ctl = (B.nlp * 32 + kThreads - 1) / kThreads;
-  if (B.grid_ctl < 1) B.grid_ctl = 1;
 }
 
 #define SCYLLA_INSTANTIATE_BATCH(T)                                                                   \
