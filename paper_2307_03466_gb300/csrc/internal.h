@@ -259,6 +259,16 @@ struct DevSetup {
   int red_blocks;
 };
 
+// Counters of a propagation.  The rounds run without the host: each of a batch of up to
+// kPropBatch has a slot, and a round whose predecessor marked no row does nothing.
+constexpr int kPropBatch = 16;
+struct PropCtl {
+  unsigned long long conflicts, rounds;
+  struct {
+    unsigned int listed, marked;  // rows with candidates to form; whether a row is active next
+  } round[kPropBatch];
+  int fractional;  // an integer column's domain has a fractional end: no row is screened
+};
 // Device side of the round-based bound propagation (propagate.cu) on the original
 // rows and columns of a handle.
 struct PropDev {
@@ -271,16 +281,24 @@ struct PropDev {
   const int* perm;                     // position in A of each entry of A^T
   const double *lo, *hi;               // row bounds (m)
   const unsigned char* is_int;         // n
-  double *dl, *du;                     // domains (n), updated in place
+  double *dl, *du;                     // the caller's domains (n), in and out
+  double2* dom;                        // domains (n), updated in place
   double *plb, *pub;                   // one round's proposals at the rows' CSR positions
   unsigned char* state;                // per row: 0 none, 1 proposals, 2 ignored
-  unsigned long long* count;           // columns changed, conflicts, rows marked
+  int* list;                           // the round's rows with candidates, their activity
+  double2* act;                        //   bounds (finite parts) and infinite counts
+  int2* ninf;
+  unsigned char* flag;                 // per column: it got a proposal this round
+  PropCtl* ctl;
 };
 cudaError_t propagate_perm(int n, const int* t_rowptr, const int* t_rows, const int* a_rowptr, const int* a_cols,
                            int* perm, cudaStream_t st);
-// one round: row visits from `active`, then the column merge marking `active_next`
-cudaError_t propagate_round(const PropDev& P, const unsigned char* active, unsigned char* active_next,
+// start of a call (every row in `active`); round `slot` of a batch: row visits from
+// `active`, then the column merge marking `active_next`; the domains back into dl and du
+cudaError_t propagate_start(const PropDev& P, unsigned char* active, cudaStream_t st);
+cudaError_t propagate_round(const PropDev& P, int slot, const unsigned char* active, unsigned char* active_next,
                             cudaStream_t st);
+cudaError_t propagate_end(const PropDev& P, cudaStream_t st);
 
 // ---- set-up launchers (setup.cu) ---------------------------------------------
 // R = C = 1, ruiz_iters Ruiz iterations and the Pock-Chambolle step (R2, C2 scratch)
@@ -428,6 +446,8 @@ template <typename T>
 cudaError_t launch_batch_part(const DevBatch<T>& B, int part, cudaStream_t st);
 template <typename T>
 cudaError_t launch_batch_get_x(const DevBatch<T>& B, int b, int col0, int count, double* out, cudaStream_t st);
+template <typename T>
+cudaError_t launch_batch_get_y(const DevBatch<T>& B, int b, int row0, int count, double* out, cudaStream_t st);
 template <typename T>
 cudaError_t launch_batch_init_point(const DevBatch<T>& B, cudaStream_t st);
 template <typename T>

@@ -882,8 +882,8 @@ void scylla_lp::set_qp_active(bool on) {
 void scylla_lp::release() {
   if (prop_mem) cudaFree(prop_mem);
   prop_mem = nullptr;
-  if (prop_count_h) cudaFreeHost(prop_count_h);
-  prop_count_h = nullptr;
+  if (prop_ctl_h) cudaFreeHost(prop_ctl_h);
+  prop_ctl_h = nullptr;
   if (repair_lp) {
     cudaStreamSynchronize(repair_lp->st);
     repair_lp->release();
@@ -1409,7 +1409,7 @@ constexpr int64_t kRepairPropagationRounds = 1000;
 
 // the buffers of the device propagation, allocated and filled on first use: perm over
 // the transpose's entries, proposals at A's positions, domains, row states, two
-// active-row masks, three counters.  The handle takes them only once every step has
+// active-row masks, the round's list, the counters.  The handle takes them only once every step has
 // succeeded, so a failed first call leaves nothing half set up.
 static int ensure_prop_buffers(scylla_lp* lp) {
   if (lp->prop_mem) return SCYLLA_OK;
@@ -1425,11 +1425,13 @@ static int ensure_prop_buffers(scylla_lp* lp) {
                o_pub = take(sizeof(double) * (nnz + 1)), o_dl = take(sizeof(double) * size_t(n0 + 1)),
                o_du = take(sizeof(double) * size_t(n0 + 1)), o_st = take(size_t(m0 + 1)),
                o_a0 = take(size_t(m0 + 1)), o_a1 = take(size_t(m0 + 1)),
-               o_cnt = take(3 * sizeof(unsigned long long));
+               o_dom = take(2 * sizeof(double) * size_t(n0 + 1)), o_list = take(sizeof(int) * size_t(m0 + 1)),
+               o_act = take(2 * sizeof(double) * size_t(m0 + 1)), o_ninf = take(2 * sizeof(int) * size_t(m0 + 1)),
+               o_flag = take(size_t(n0 + 1)), o_ctl = take(sizeof(PropCtl));
   void* mem = nullptr;
-  unsigned long long* count_h = nullptr;
+  PropCtl* ctl_h = nullptr;
   cudaError_t e = cudaMalloc(&mem, off);
-  if (e == cudaSuccess) e = cudaMallocHost(&count_h, 3 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMallocHost(&ctl_h, sizeof(PropCtl));
   PropDev P{};
   if (e == cudaSuccess) {
     char* b = static_cast<char*>(mem);
@@ -1448,13 +1450,18 @@ static int ensure_prop_buffers(scylla_lp* lp) {
     P.dl = reinterpret_cast<double*>(b + o_dl);
     P.du = reinterpret_cast<double*>(b + o_du);
     P.state = reinterpret_cast<unsigned char*>(b + o_st);
-    P.count = reinterpret_cast<unsigned long long*>(b + o_cnt);
+    P.dom = reinterpret_cast<double2*>(b + o_dom);
+    P.list = reinterpret_cast<int*>(b + o_list);
+    P.act = reinterpret_cast<double2*>(b + o_act);
+    P.ninf = reinterpret_cast<int2*>(b + o_ninf);
+    P.flag = reinterpret_cast<unsigned char*>(b + o_flag);
+    P.ctl = reinterpret_cast<PropCtl*>(b + o_ctl);
     e = propagate_perm(int(n0), lp->t_rowptr, lp->t_cols, lp->a_rowptr, lp->a_cols, perm, lp->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(lp->st);
   }
   if (e != cudaSuccess) {
     if (mem) cudaFree(mem);
-    if (count_h) cudaFreeHost(count_h);
+    if (ctl_h) cudaFreeHost(ctl_h);
     set_error(std::string("device propagation buffers: ") + cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? SCYLLA_ERR_OOM : SCYLLA_ERR_CUDA;
   }
@@ -1462,7 +1469,7 @@ static int ensure_prop_buffers(scylla_lp* lp) {
   lp->prop = P;
   lp->prop_active[0] = reinterpret_cast<unsigned char*>(b + o_a0);
   lp->prop_active[1] = reinterpret_cast<unsigned char*>(b + o_a1);
-  lp->prop_count_h = count_h;
+  lp->prop_ctl_h = ctl_h;
   lp->prop_mem = mem;
   return SCYLLA_OK;
 }
@@ -1480,21 +1487,24 @@ static int propagate_impl(scylla_lp* lp, double* dl, double* du, uint8_t* ignore
   P.hi = lp->hi_un;
   CK(cudaMemcpyAsync(P.dl, dl, sizeof(double) * n0, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(P.du, du, sizeof(double) * n0, cudaMemcpyHostToDevice, st));
-  if (m0 > 0) {
-    CK(cudaMemsetAsync(P.state, 0, size_t(m0), st));
-    CK(cudaMemsetAsync(lp->prop_active[0], 1, size_t(m0), st));
-  }
+  CK(propagate_start(P, lp->prop_active[0], st));
+  // The host looks at the counters after 4, 8, 16, 16, ... rounds (most calls end within
+  // the first few; a round past the end costs three launches that return at once).
   int64_t rounds = 0, conflicts = 0;
-  int cur = 0;
-  while (m0 > 0 && rounds < max_rounds) {
-    ++rounds;
-    CK(propagate_round(P, lp->prop_active[cur], lp->prop_active[cur ^ 1], st));
-    CK(cudaMemcpyAsync(lp->prop_count_h, P.count, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+  int cur = 0, batch = 4;
+  for (int64_t done = 0; m0 > 0 && done < max_rounds; batch = std::min(2 * batch, kPropBatch)) {
+    const int count = int(std::min<int64_t>(batch, max_rounds - done));
+    for (int s = 0; s < count; ++s, cur ^= 1)
+      CK(propagate_round(P, s, lp->prop_active[cur], lp->prop_active[cur ^ 1], st));
+    CK(cudaMemcpyAsync(lp->prop_ctl_h, P.ctl, sizeof(PropCtl), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    conflicts += int64_t(lp->prop_count_h[1]);
-    if (lp->prop_count_h[2] == 0) break;  // no row is active next
-    cur ^= 1;
+    done += count;
+    rounds = int64_t(lp->prop_ctl_h->rounds);
+    conflicts = int64_t(lp->prop_ctl_h->conflicts);
+    if (lp->prop_ctl_h->round[count - 1].marked == 0u) break;  // no row is active next
+    if (done < max_rounds) CK(cudaMemsetAsync(P.ctl->round, 0, sizeof(P.ctl->round), st));
   }
+  CK(propagate_end(P, st));
   CK(cudaMemcpyAsync(dl, P.dl, sizeof(double) * n0, cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(du, P.du, sizeof(double) * n0, cudaMemcpyDeviceToHost, st));
   std::vector<unsigned char> state(static_cast<size_t>(m0));

@@ -121,7 +121,7 @@ struct scylla_lp {
   void* prop_mem = nullptr;
   scylla::PropDev prop{};
   unsigned char* prop_active[2] = {nullptr, nullptr};
-  unsigned long long* prop_count_h = nullptr;  // pinned copy of the three counters
+  scylla::PropCtl* prop_ctl_h = nullptr;  // pinned copy of its counters
 
   scylla::DevObjective objective_desc();
   void release();

@@ -48,46 +48,107 @@ __global__ void k_prop_perm(int n, const int* __restrict__ t_rowptr, const int* 
   }
 }
 
-// one round's row visits.  state[i]: 0 no proposals this round, 1 proposals in
-// plb/pub at the row's CSR positions (-inf / +inf where a bound is not tightened),
-// 2 ignored for good
+// the caller's domains side by side, and whether an integer column's is fractional (then
+// no row is screened: the rounding alone changes such a bound)
+__global__ void k_prop_in(PropDev P) {
+  bool frac = false;
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < P.n; j += gridDim.x * blockDim.x) {
+    const double l = P.dl[j], u = P.du[j];
+    P.dom[j] = make_double2(l, u);
+    frac = frac || (P.is_int[j] && (l != floor(l) || u != floor(u)));
+  }
+  if (frac) P.ctl->fractional = 1;
+}
+__global__ void k_prop_out(PropDev P) {
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < P.n; j += gridDim.x * blockDim.x) {
+    const double2 d = P.dom[j];
+    P.dl[j] = d.x;
+    P.du[j] = d.y;
+  }
+}
+
+__device__ __forceinline__ bool prop_inf(double v) {
+  return (__double_as_longlong(v) & 0x7fffffffffffffffLL) == 0x7ff0000000000000LL;
+}
+
+// Whether a round has anything to do: the first of a call, or its predecessor marked a row.
+__device__ __forceinline__ bool prop_on(const PropCtl* c, int slot) { return slot == 0 || c->round[slot - 1].marked != 0u; }
+
+// One round, first half: the activity bounds of every active row (one thread per row, in
+// CSR order).  A row whose sides' slacks both exceed its largest single-column span
+// |a_j| (u_j - l_j) by a relative margin of 1e-6 cannot change a domain: its visit ends
+// here, without the divisions of the candidates (95% of the visits of the packing/covering
+// workload; the whole propagation was bound by them).  The others go on a list for the
+// second half.  state[i]: 0 no proposals this round, 1 proposals in plb/pub at the row's
+// CSR positions (-inf / +inf where a bound is not tightened), 2 ignored for good.
 __global__ void __launch_bounds__(kPropThreads)
-    k_prop_rows(PropDev P, const unsigned char* __restrict__ active) {
+    k_prop_rows(PropDev P, int slot, const unsigned char* __restrict__ active, unsigned char* __restrict__ active_next) {
+  PropCtl* ctl = P.ctl;
+  if (!prop_on(ctl, slot)) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) ++ctl->rounds;
   const double inf = __longlong_as_double(0x7ff0000000000000LL);
+  const bool screen = ctl->fractional == 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.m; i += gridDim.x * blockDim.x) {
-    if (P.state[i] == 2) continue;
-    if (!active[i]) {
-      P.state[i] = 0;
-      continue;
-    }
+    active_next[i] = 0;
+    const unsigned char st = P.state[i];
+    if (st == 2) continue;
+    if (st != 0) P.state[i] = 0;
+    if (!active[i]) continue;
     const double lo_i = P.lo[i], hi_i = P.hi[i];
-    if (lo_i == -inf && hi_i == inf) {
-      P.state[i] = 0;
-      continue;
-    }
+    if (lo_i == -inf && hi_i == inf) continue;
     const int p0 = P.rowptr[i], p1 = P.rowptr[i + 1];
-    double minf = 0.0, maxf = 0.0;
+    double minf = 0.0, maxf = 0.0, span = 0.0;
     int nmin = 0, nmax = 0;
+    bool zero = false;
     for (int p = p0; p < p1; ++p) {
-      const int j = P.cols[p];
       const double a = P.vals[p];
-      const double bmin = a > 0.0 ? P.dl[j] : P.du[j];
-      const double bmax = a > 0.0 ? P.du[j] : P.dl[j];
-      if (isinf(bmin)) ++nmin;
+      const double2 d = P.dom[P.cols[p]];
+      const bool pos = __double_as_longlong(a) > 0;
+      const double bmin = pos ? d.x : d.y, bmax = pos ? d.y : d.x;
+      if (prop_inf(bmin)) ++nmin;
       else minf = __dadd_rn(minf, __dmul_rn(a, bmin));
-      if (isinf(bmax)) ++nmax;
+      if (prop_inf(bmax)) ++nmax;
       else maxf = __dadd_rn(maxf, __dmul_rn(a, bmax));
+      span = fmax(span, fabs(a) * (d.y - d.x));
+      zero = zero || a == 0.0;
     }
     if ((nmin == 0 && hi_i != inf && minf > __dadd_rn(hi_i, 1e-9)) ||
         (nmax == 0 && lo_i != -inf && maxf < __dsub_rn(lo_i, 1e-9))) {
       P.state[i] = 2;
       continue;
     }
+    constexpr double kMarg = 1e-6;
+    const bool hi_side = hi_i != inf && (nmin == 1 || (nmin == 0 && !((hi_i - minf) > span * (1.0 + kMarg) +
+                                                       kMarg * (1.0 + fabs(hi_i) + fabs(minf)))));
+    const bool lo_side = lo_i != -inf && (nmax == 1 || (nmax == 0 && !((maxf - lo_i) > span * (1.0 + kMarg) +
+                                                        kMarg * (1.0 + fabs(lo_i) + fabs(maxf)))));
+    if (screen && !zero && !hi_side && !lo_side) continue;
+    P.act[i] = make_double2(minf, maxf);
+    P.ninf[i] = make_int2(nmin, nmax);
+    P.list[atomicAdd(&ctl->round[slot].listed, 1u)] = i;
+  }
+}
+
+// Second half: the candidates of the listed rows, a warp per row, a lane per entry.  The
+// columns that get a proposal are flagged for the merge.
+__global__ void __launch_bounds__(kPropThreads) k_prop_visit(PropDev P, int slot) {
+  PropCtl* ctl = P.ctl;
+  if (!prop_on(ctl, slot)) return;
+  const double inf = __longlong_as_double(0x7ff0000000000000LL);
+  const int lane = threadIdx.x & 31, count = int(ctl->round[slot].listed);
+  for (int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < count; v += (gridDim.x * blockDim.x) >> 5) {
+    const int i = P.list[v];
+    const double lo_i = P.lo[i], hi_i = P.hi[i];
+    const double2 act = P.act[i];
+    const int2 ni = P.ninf[i];
+    const double minf = act.x, maxf = act.y;
+    const int nmin = ni.x, nmax = ni.y, p1 = P.rowptr[i + 1];
     bool ignore = false;
-    for (int p = p0; p < p1; ++p) {
+    for (int p = P.rowptr[i] + lane; p < p1; p += 32) {
       const int j = P.cols[p];
       const double a = P.vals[p];
-      const double old_lb = P.dl[j], old_ub = P.du[j];
+      const double2 d = P.dom[j];
+      const double old_lb = d.x, old_ub = d.y;
       const double bmin = a > 0.0 ? old_lb : old_ub;
       const double bmax = a > 0.0 ? old_ub : old_lb;
       double rmin, rmax;
@@ -109,12 +170,12 @@ __global__ void __launch_bounds__(kPropThreads)
       double new_lb = old_lb, new_ub = old_ub;
       if (P.is_int[j]) {
         if (cand_ub != inf) {
-          const double v = floor(__dadd_rn(cand_ub, 1e-6));
-          if (v < old_ub) new_ub = v;
+          const double v2 = floor(__dadd_rn(cand_ub, 1e-6));
+          if (v2 < old_ub) new_ub = v2;
         }
         if (cand_lb != -inf) {
-          const double v = ceil(__dsub_rn(cand_lb, 1e-6));
-          if (v > old_lb) new_lb = v;
+          const double v2 = ceil(__dsub_rn(cand_lb, 1e-6));
+          if (v2 > old_lb) new_lb = v2;
         }
       } else {
         if (cand_ub != inf &&
@@ -124,28 +185,29 @@ __global__ void __launch_bounds__(kPropThreads)
             (old_lb == -inf || cand_lb > __dadd_rn(old_lb, __dmul_rn(1e-3, fmax(1.0, fabs(old_lb))))))
           new_lb = cand_lb;
       }
-      if (new_lb != old_lb || new_ub != old_ub) {
-        if (new_lb > __dadd_rn(new_ub, 1e-9)) {
-          ignore = true;
-          break;
-        }
-      }
+      const bool moved = new_lb != old_lb || new_ub != old_ub;
+      if (moved && new_lb > __dadd_rn(new_ub, 1e-9)) ignore = true;
       P.plb[p] = new_lb != old_lb ? new_lb : -inf;
       P.pub[p] = new_ub != old_ub ? new_ub : inf;
+      if (moved) P.flag[j] = 1;
     }
-    P.state[i] = ignore ? 2 : 1;
+    ignore = __any_sync(0xffffffffu, ignore);
+    if (lane == 0) P.state[i] = ignore ? 2 : 1;
   }
 }
 
-// the merge of one round: each column over its rows' proposals; changed columns
-// mark their rows active for the next round.  count[0]: columns changed, count[1]:
-// conflicts, count[2]: set when a row was marked
+// The merge of one round: each flagged column over its rows' proposals; changed columns
+// mark their rows active for the next round.
 __global__ void __launch_bounds__(kPropThreads)
-    k_prop_cols(PropDev P, unsigned char* __restrict__ active_next) {
+    k_prop_cols(PropDev P, int slot, unsigned char* __restrict__ active_next) {
+  PropCtl* ctl = P.ctl;
+  if (!prop_on(ctl, slot)) return;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < P.n; j += gridDim.x * blockDim.x) {
+    if (!P.flag[j]) continue;
+    P.flag[j] = 0;
     const int q0 = P.t_rowptr[j], q1 = P.t_rowptr[j + 1];
-    const double ol = P.dl[j], ou = P.du[j];
-    double nl = ol, nu = ou;
+    const double2 d = P.dom[j];
+    double nl = d.x, nu = d.y;
     for (int q = q0; q < q1; ++q) {
       const int i = P.t_rows[q];
       if (i >= P.m || P.state[i] != 1) continue;
@@ -153,14 +215,12 @@ __global__ void __launch_bounds__(kPropThreads)
       nl = fmax(nl, P.plb[p]);
       nu = fmin(nu, P.pub[p]);
     }
-    if (nl == ol && nu == ou) continue;
+    if (nl == d.x && nu == d.y) continue;
     if (nl > __dadd_rn(nu, 1e-9)) {
-      atomicAdd(P.count + 1, 1ULL);
+      atomicAdd(&ctl->conflicts, 1ULL);
       continue;
     }
-    P.dl[j] = nl;
-    P.du[j] = nu;
-    atomicAdd(P.count, 1ULL);
+    P.dom[j] = make_double2(nl, nu);
     bool marked = false;
     for (int q = q0; q < q1; ++q) {
       const int i = P.t_rows[q];
@@ -168,7 +228,7 @@ __global__ void __launch_bounds__(kPropThreads)
       active_next[i] = 1;
       marked = true;
     }
-    if (marked) atomicOr(reinterpret_cast<unsigned long long*>(P.count + 2), 1ULL);
+    if (marked) ctl->round[slot].marked = 1u;
   }
 }
 
@@ -180,13 +240,28 @@ cudaError_t propagate_perm(int n, const int* t_rowptr, const int* t_rows, const 
   return cudaGetLastError();
 }
 
-cudaError_t propagate_round(const PropDev& P, const unsigned char* active, unsigned char* active_next,
-                            cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(active_next, 0, size_t(P.m > 0 ? P.m : 1), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(P.count, 0, 3 * sizeof(unsigned long long), st);
+cudaError_t propagate_start(const PropDev& P, unsigned char* active, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(P.ctl, 0, sizeof(PropCtl), st);
+  if (e == cudaSuccess && P.m > 0) e = cudaMemsetAsync(P.state, 0, size_t(P.m), st);
+  if (e == cudaSuccess && P.m > 0) e = cudaMemsetAsync(active, 1, size_t(P.m), st);
+  if (e == cudaSuccess && P.n > 0) e = cudaMemsetAsync(P.flag, 0, size_t(P.n), st);
   if (e != cudaSuccess) return e;
-  if (P.m > 0) k_prop_rows<<<prop_grid(P.m), kPropThreads, 0, st>>>(P, active);
-  if (P.n > 0) k_prop_cols<<<prop_grid(P.n), kPropThreads, 0, st>>>(P, active_next);
+  if (P.n > 0) k_prop_in<<<prop_grid(P.n), kPropThreads, 0, st>>>(P);
+  return cudaGetLastError();
+}
+
+cudaError_t propagate_round(const PropDev& P, int slot, const unsigned char* active, unsigned char* active_next,
+                            cudaStream_t st) {
+  if (P.m > 0) {
+    k_prop_rows<<<prop_grid(P.m), kPropThreads, 0, st>>>(P, slot, active, active_next);
+    k_prop_visit<<<prop_grid(32LL * P.m), kPropThreads, 0, st>>>(P, slot);
+  }
+  if (P.n > 0) k_prop_cols<<<prop_grid(P.n), kPropThreads, 0, st>>>(P, slot, active_next);
+  return cudaGetLastError();
+}
+
+cudaError_t propagate_end(const PropDev& P, cudaStream_t st) {
+  if (P.n > 0) k_prop_out<<<prop_grid(P.n), kPropThreads, 0, st>>>(P);
   return cudaGetLastError();
 }
 
