@@ -42,7 +42,7 @@ struct scylla_batch {
   size_t arena_bytes = 0;
   std::vector<Control> ctl0;  // control blocks at create (cold restart)
   Control* h_ctl = nullptr;   // pinned mirror of the control array
-  double* io = nullptr;       // device staging for primal output
+  double* io = nullptr;       // device staging for primal and dual output
   DevBatch<double> b64{};
   DevBatch<float> b32{};
   cudaGraph_t graph = nullptr;
@@ -126,11 +126,15 @@ int batch_solve_persistent(scylla_batch* h, DevBatch<T>& B, double tol, int64_t 
   CKB(cudaMemcpyAsync(&h->h_done[1], B.n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
   CKB(cudaStreamSynchronize(st));
   if (h->h_done[1] < h->nlp) {
+    // the check at the iteration limit ends the solve, so no chunk is queued ahead past it
+    const long long need = (iter_limit + nchk - 1) / nchk;
     CKB(enqueue(0));
     for (long long c = 0; c < max_chunks; ++c) {
-      if (c + 1 < max_chunks) CKB(enqueue(c + 1));
+      const bool ahead = c + 1 < need;
+      if (ahead) CKB(enqueue(c + 1));
       CKB(cudaEventSynchronize(h->ev_chunk[c & 1]));
       if (h->h_done[c & 1] >= h->nlp) break;
+      if (!ahead && c + 1 < max_chunks) CKB(enqueue(c + 1));
     }
   }
   CKB(cudaEventRecord(h->ev1, st));
@@ -212,11 +216,15 @@ int batch_solve_impl(scylla_batch* h, DevBatch<T>& B, double tol, int64_t iter_l
   CKB(cudaMemcpyAsync(&h->h_done[1], B.n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
   CKB(cudaStreamSynchronize(st));
   if (h->h_done[1] < h->nlp) {
+    // the check at the iteration limit ends the solve, so no chunk is queued ahead past it
+    const long long need = (iter_limit + nchk - 1) / nchk;
     CKB(enqueue(0));
     for (long long c = 0; c < max_chunks; ++c) {
-      if (c + 1 < max_chunks) CKB(enqueue(c + 1));
+      const bool ahead = c + 1 < need;
+      if (ahead) CKB(enqueue(c + 1));
       CKB(cudaEventSynchronize(h->ev_chunk[c & 1]));
       if (h->h_done[c & 1] >= h->nlp) break;
+      if (!ahead && c + 1 < max_chunks) CKB(enqueue(c + 1));
     }
   }
   CKB(cudaEventRecord(h->ev1, st));
@@ -421,7 +429,7 @@ int create_batch(int32_t count, const scylla_csr* A, const double* const* c, con
     q_ctr = ar.take<unsigned int>(4);
     lp_cnt = ar.take<unsigned int>(count);
     gbar = ar.take<char>(16);
-    h->io = ar.take<double>(n);
+    h->io = ar.take<double>(std::max(n, m));  // primal or dual of one LP
     if (pass == 0) h->arena_bytes = ar.off + 256;
   }
   cudaStream_t st = h->st;
@@ -775,8 +783,7 @@ extern "C" int scylla_batch_get_primal(const scylla_batch* h, int32_t b, double*
 }
 
 // y of LP b from its current pool (the pair a finished LP returns, whose errors its
-// result reports), unscaled on the host: y_i = y~_i R_i in FP64, as the primal's
-// getter does on the device
+// result reports), unscaled on the device as the primal's
 extern "C" int scylla_batch_get_dual(const scylla_batch* h, int32_t b, double* y) {
   if (!h || !y || b < 0 || b >= h->nlp) {
     set_error("invalid argument");
@@ -785,28 +792,10 @@ extern "C" int scylla_batch_get_dual(const scylla_batch* h, int32_t b, double* y
   const int r0 = h->row_off[b], cnt = h->row_off[b + 1] - h->row_off[b];
   if (cnt == 0) return SCYLLA_OK;
   cudaStream_t st = h->st;
-  const bool mixed = h->p.precision == SCYLLA_PREC_MIXED;
-  const Control* dctl = mixed ? h->b32.ctl : h->b64.ctl;
-  int cur = -1;
-  CKB(cudaMemcpyAsync(&cur, &dctl[b].ix_cur, sizeof(int), cudaMemcpyDeviceToHost, st));
+  if (h->p.precision == SCYLLA_PREC_MIXED) CKB(launch_batch_get_y<float>(h->b32, b, r0, cnt, h->io, st));
+  else CKB(launch_batch_get_y<double>(h->b64, b, r0, cnt, h->io, st));
+  CKB(cudaMemcpyAsync(y, h->io, sizeof(double) * size_t(cnt), cudaMemcpyDeviceToHost, st));
   CKB(cudaStreamSynchronize(st));
-  if (cur < 0 || cur > 2) {
-    set_error("pool index out of range");
-    return SCYLLA_ERR_CUDA;
-  }
-  std::vector<double> R(static_cast<size_t>(cnt));
-  const double* Rd = mixed ? h->b32.d.R : h->b64.d.R;
-  CKB(cudaMemcpyAsync(R.data(), Rd + r0, sizeof(double) * size_t(cnt), cudaMemcpyDeviceToHost, st));
-  if (mixed) {
-    std::vector<float> v(static_cast<size_t>(cnt));
-    CKB(cudaMemcpyAsync(v.data(), h->b32.d.Y[cur] + r0, sizeof(float) * size_t(cnt), cudaMemcpyDeviceToHost, st));
-    CKB(cudaStreamSynchronize(st));
-    for (int i = 0; i < cnt; ++i) y[i] = double(v[size_t(i)]) * R[size_t(i)];
-  } else {
-    CKB(cudaMemcpyAsync(y, h->b64.d.Y[cur] + r0, sizeof(double) * size_t(cnt), cudaMemcpyDeviceToHost, st));
-    CKB(cudaStreamSynchronize(st));
-    for (int i = 0; i < cnt; ++i) y[i] *= R[size_t(i)];
-  }
   return SCYLLA_OK;
 }
 

@@ -881,6 +881,37 @@ static __device__ void check_control_warp(Control* c, const double* r, double* t
   __syncwarp();
 }
 
+// a control block into a warp's shared copy (L2 loads) and back, word by word
+__device__ __forceinline__ void ctl_in(Control* dst, const Control* src) {
+  static_assert(sizeof(Control) % 4 == 0, "word copy");
+  const int lane = threadIdx.x & 31;
+  for (int i = lane; i < int(sizeof(Control) / 4); i += 32)
+    reinterpret_cast<int*>(dst)[i] = __ldcg(reinterpret_cast<const int*>(src) + i);
+  __syncwarp();
+}
+__device__ __forceinline__ void ctl_out(Control* dst, const Control* src) {
+  __syncwarp();
+  const int lane = threadIdx.x & 31;
+  for (int i = lane; i < int(sizeof(Control) / 4); i += 32)
+    reinterpret_cast<int*>(dst)[i] = reinterpret_cast<const int*>(src)[i];
+  __syncwarp();
+}
+
+// One lane's chain of partial sums part[t * stride + off], t = beg, beg + step, ... <
+// end, added in that order; eight loads in flight.
+__device__ __forceinline__ double chain_sum(const double* part, int stride, int off, int beg, int end, int step) {
+  double v = 0.0;
+  for (int t = beg; t < end; t += 8 * step) {
+    double x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = t + u * step < end ? __ldcg(part + size_t(t + u * step) * stride + off) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (t + u * step < end) v += x[u];
+  }
+  return v;
+}
+
 // per-thread accumulator type of the bulk kernels
 template <typename T>
 struct AccOf {

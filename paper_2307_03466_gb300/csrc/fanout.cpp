@@ -114,11 +114,15 @@ int fan_solve_impl(scylla_fanout* f, DevFan<T>& F, double tol, int64_t iter_limi
   CKF(cudaMemcpyAsync(&f->h_done[1], F.n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
   CKF(cudaStreamSynchronize(st));
   if (f->h_done[1] < f->K) {
+    // the check at the iteration limit ends the solve, so no chunk is queued ahead past it
+    const long long need = (iter_limit + nchk - 1) / nchk;
     CKF(enqueue(0));
     for (long long c = 0; c < max_chunks; ++c) {
-      if (c + 1 < max_chunks) CKF(enqueue(c + 1));
+      const bool ahead = c + 1 < need;
+      if (ahead) CKF(enqueue(c + 1));
       CKF(cudaEventSynchronize(f->ev_chunk[c & 1]));
       if (f->h_done[c & 1] >= f->K) break;
+      if (!ahead && c + 1 < max_chunks) CKF(enqueue(c + 1));
     }
   }
   CKF(cudaEventRecord(f->ev1, st));

@@ -39,7 +39,8 @@ constexpr int kFWarps = kFThreads / 32;
 
 __device__ __forceinline__ double fwarp_sum(double v) { return warp_sum(v); }
 
-// sum over the row's nonzeros of a_rp * src[col][k] for the lane's two objectives;
+// sums over the row's nonzeros of a_rp * src[col] for two vectors per lane (the checks:
+// the current and the averaged point of the lane's objective);
 // the (index, value) pairs are loaded 32 at a time and broadcast by shuffles, four
 // nonzeros per step so eight gathers per lane are in flight.  Lanes past the row end
 // carry (column 0, value 0), which adds exactly zero, so the four-wide steps need
@@ -134,7 +135,7 @@ __device__ __forceinline__ void row_gather_pair(int p0, int p1, const int* __res
   }
 }
 
-// A check's products of one row for the lane's two objectives: out in FP64 for the
+// A check's products of one row for the two points of the lane's objective: out in FP64 for the
 // check's sums, ref in the iterates' precision for the refresh of the cached products
 // (FP64: the FP64 sums; FP32-mixed: the FP32 pairs of row_gather_pair, ref their
 // rounded value).  src(col, g) gives the two gathered entries in T.
@@ -157,18 +158,25 @@ __device__ __forceinline__ void check_gather(int p0, int p1, const int* __restri
   }
 }
 
-template <typename T>
-__device__ __forceinline__ void store_block_sums(const typename AccOf<T>::type* acc /*[2][N]*/, int N, double* part,
-                                                 double* sh /*[kFWarps][N*kFK]*/) {
-  // per objective and sum: warp partials to shared memory, then block sums
+// Halves of the 64 slots that the objectives take: a check's warp works on one half of
+// one row, so fan-outs of up to 32 objectives skip the other.
+__device__ __forceinline__ int fan_halves(int K) { return K > 32 ? 2 : 1; }
+
+// block sums of the checks' per-lane accumulators into part[block][sum][objective]: warp
+// w holds the half w % halves, lane l its objective l
+template <int N>
+__device__ __forceinline__ void store_block_sums(const double (&acc)[N], int halves, double* part,
+                                                 double* sh /*[kFWarps][N][32]*/) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int q = 0; q < 2; ++q)
-    for (int s = 0; s < N; ++s) sh[(w * N + s) * kFK + lane + 32 * q] = double(acc[q * N + s]);
+#pragma unroll
+  for (int s = 0; s < N; ++s) sh[(w * N + s) * 32 + lane] = acc[s];
   __syncthreads();
   for (int idx = threadIdx.x; idx < N * kFK; idx += blockDim.x) {
+    const int s = idx / kFK, k = idx % kFK;
     double t = 0.0;
-    for (int v = 0; v < kFWarps; ++v) t += sh[v * N * kFK + idx];
-    part[blockIdx.x * N * kFK + idx] = t;  // [block][sum][objective]
+    if (k < 32 * halves)
+      for (int v = k / 32; v < kFWarps; v += halves) t += sh[(v * N + s) * 32 + (k & 31)];
+    part[size_t(blockIdx.x) * N * kFK + idx] = t;
   }
 }
 
@@ -453,6 +461,7 @@ template <typename T, int VEC, int CHUNK>
 __global__ void __launch_bounds__(kFThreads, sizeof(T) == 4 ? 4 : 3) k_fprimal(DevFan<T> F) {
   typedef typename AccOf<T>::type A;
   typedef FanGeo<VEC, CHUNK> G;
+  if (*F.n_done >= F.K) return;
   __shared__ double sh[kFWarps * 1 * kFK];
   __shared__ __align__(16) FanShared<T> S;
   load_fan_shared(F, S);
@@ -580,6 +589,7 @@ template <typename T, int VEC, int CHUNK>
 __global__ void __launch_bounds__(kFThreads, sizeof(T) == 4 && !(VEC == 4 && CHUNK == 32) ? 4 : 3) k_fdual(DevFan<T> F) {
   typedef typename AccOf<T>::type A;
   typedef FanGeo<VEC, CHUNK> G;
+  if (*F.n_done >= F.K) return;
   __shared__ double sh[kFWarps * 2 * kFK];
   __shared__ __align__(16) FanShared<T> S;
   __shared__ __align__(16) FanStage<T, VEC> E;
@@ -739,21 +749,23 @@ __device__ __forceinline__ void write_fan_slot(FanSlot<T>* s, const Control* c) 
   *s = v;
 }
 
-// One warp per objective: block sums in a fixed order, then the step decision;
-// rej[k] says whether objective k's attempt was rejected (k_fcopy_rej restores its
-// pair).  Block 0 counts the attempt, which swaps the pool roles of every objective.
+// A block per objective: block sums in a fixed order (a warp per sum, eight loads in
+// flight), then the step decision on a shared copy of the control block; rej[k] says
+// whether objective k's attempt was rejected (k_fcopy_rej restores its pair).  Block 0
+// counts the attempt, which swaps the pool roles of every objective.
+constexpr int kFStepThreads = 3 * 32;
 template <typename T>
-__global__ void __launch_bounds__(kFThreads) k_fstep_control(DevFan<T> F) {
+__global__ void __launch_bounds__(kFStepThreads) k_fstep_control(DevFan<T> F) {
+  if (*F.n_done >= F.K) return;  // nothing attempted: the pools keep their roles
   FanState* st = F.state;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ++*F.kglob;
     ++st->att;
   }
-  const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (k >= F.K) return;
+  const int k = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int flags = F.slot[k].flags;
   if (!(flags & kSlotActive)) {
-    if (lane == 0) {
+    if (threadIdx.x == 0) {
       st->rej[k] = 0;
       if (flags & kSlotCheck) {  // carried: the pending average update is now applied
         Control* c = &F.ctl[k];
@@ -767,30 +779,27 @@ __global__ void __launch_bounds__(kFThreads) k_fstep_control(DevFan<T> F) {
     }
     return;
   }
-  const int G = F.grid_p, H = F.grid_d;
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-  // the partials are [sum][objective][block]: a warp's loads are consecutive
-  const double* pp = F.part_p + size_t(k) * G;
-  const double* pd0 = F.part_d + size_t(k) * H;
-  const double* pd1 = F.part_d + size_t(kFK + k) * H;
-  for (int b = lane; b < G; b += 32) s0 += pp[b];
-  for (int b = lane; b < H; b += 32) {
-    s1 += pd0[b];
-    s2 += pd1[b];
+  __shared__ Control sc;
+  __shared__ double red[3];
+  if (w == 2) ctl_in(&sc, F.ctl + k);
+  {
+    // the partials are [sum][objective][block]: a warp's loads are consecutive
+    const double* p = w == 0 ? F.part_p + size_t(k) * F.grid_p : F.part_d + size_t((w - 1) * kFK + k) * F.grid_d;
+    const double s = fwarp_sum(chain_sum(p, 1, 0, lane, w == 0 ? F.grid_p : F.grid_d, 32));
+    if (lane == 0) red[w] = s;
   }
-  s0 = fwarp_sum(s0);
-  s1 = fwarp_sum(s1);
-  s2 = fwarp_sum(s2);
+  __syncthreads();
+  if (w != 0) return;
   if (lane == 0) {
-    Control* c = &F.ctl[k];
+    Control* c = &sc;
     const long long rej0 = c->rejected;
     if constexpr (sizeof(T) == 4) {
       // FP32-mixed: the single-LP path's FP32 decision (no FP64 division on the
       // per-attempt path); the FP64 sums are rounded once
       const StepPre p = step_pre<float>(c, F.d.step_fac, F.d.n_check);
-      step_control<float>(c, p, float(s0), float(s1), float(s2), nullptr, 0);
+      step_control<float>(c, p, float(red[0]), float(red[1]), float(red[2]), nullptr, 0);
     } else {
-      step_control(c, s0, s1, s2, F.d.step_fac, F.d.n_check, nullptr, 0);
+      step_control(c, red[0], red[1], red[2], F.d.step_fac, F.d.n_check, nullptr, 0);
     }
     st->rej[k] = c->rejected != rej0 ? 1 : 0;
     if (c->done) atomicAdd(F.n_done, 1);
@@ -799,231 +808,201 @@ __global__ void __launch_bounds__(kFThreads) k_fstep_control(DevFan<T> F) {
     // restored by k_fcopy_rej) gathers it again
     F.slot[k].flags &= ~kSlotCached;
   }
+  ctl_out(F.ctl + k, &sc);
 }
 
 // Column half of a check for every objective: A^T y of the current and the averaged
 // dual (FP64 sums, or in FP32-mixed the FP32 pairs of check_gather), reduced costs
-// against c_hat_k, residuals, objectives, hash, all in FP64.  Lane q of a warp works
-// on objectives q and q + 32 of one column.  FP32 entries widen to FP64 by the exact
-// bit-level conversion on the integer pipe (an FP32-to-FP64 conversion instruction
-// would take the FP64 pipe, the bound of these kernels on this part).
+// against c_hat_k, residuals, objectives, hash, all in FP64.  A warp works on one half of
+// the objectives of one column, a lane on both points of one objective, so one walk over
+// the column serves both (the walk's loads, the splitting of its values and their
+// broadcasts), and a lane holds ten FP64 accumulators, not twenty (three blocks per SM
+// resident instead of two).  FP32 entries widen to FP64 by the exact bit-level conversion
+// on the integer pipe (an FP32-to-FP64 conversion instruction would take the FP64 pipe,
+// the bound of these kernels on this part).
 template <typename T>
-__global__ void __launch_bounds__(kFThreads) k_fcheck_cols(DevFan<T> F) {
-  __shared__ double sh[kFWarps * kNC1 * kFK];
-  const int lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(kFThreads, 3) k_fcheck_cols(DevFan<T> F) {
+  if (*F.n_done >= F.K) return;
+  __shared__ double sh[kFWarps * kNC1 * 32];
+  const int lane = threadIdx.x & 31, halves = fan_halves(F.K);
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+  const int k = lane + 32 * (gw % halves);
   const DevLP<T>& d = F.d;
   const int cur = fan_cur(F);
-  bool on[2], hs[2];
-  int fl[2];
-  T w[2], w1[2];
+  const int fl = k < F.K ? F.slot[k].flags : 0;
+  const bool on = (fl & kSlotCheck) != 0, avg = (fl & kSlotAvg) != 0;
+  const T w = k < F.K ? F.slot[k].w : T(0), w1 = k < F.K ? F.slot[k].w1 : T(1);
+  // the hash of the rounded point only feeds the stall test
+  const bool hs = k < F.K && F.ctl[k].stall_checks > 0;
+  double acc[kNC1];
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int k = lane + 32 * q;
-    fl[q] = k < F.K ? F.slot[k].flags : 0;
-    on[q] = (fl[q] & kSlotCheck) != 0;
-    w[q] = k < F.K ? F.slot[k].w : T(0);
-    w1[q] = k < F.K ? F.slot[k].w1 : T(1);
-    // the hash of the rounded point only feeds the stall test
-    hs[q] = k < F.K && F.ctl[k].stall_checks > 0;
-  }
-  double acc[2 * kNC1];
-#pragma unroll
-  for (int q = 0; q < 2 * kNC1; ++q) acc[q] = 0.0;
-  unsigned long long h[2] = {0ULL, 0ULL};
-  const T* yc = F.Y[cur];
-  const T* ya = F.Y[2];
-  T* Xc = F.X[cur];
-  T* Xa = F.X[2];
-  for (int j = gw; j < d.n; j += nw) {
-    double sc[2], sa[2];
-    T rc[2], ra[2];
-    auto srcc = [&](int i, T(&g)[2]) {
-#pragma unroll
-      for (int q = 0; q < 2; ++q) g[q] = on[q] ? yc[size_t(i) * kFK + lane + 32 * q] : T(0);
-    };
-    auto srca = [&](int i, T(&g)[2]) {
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        if (!on[q]) {
-          g[q] = T(0);
-          continue;
-        }
-        const size_t o = size_t(i) * kFK + lane + 32 * q;
-        T v = ya[o];
-        if (fl[q] & kSlotAvg) v = blend(v, yc[o], w1[q], w[q]);
-        g[q] = v;
-      }
-    };
-    check_gather<T>(d.t_rowptr[j], d.t_rowptr[j + 1], d.t_cols, d.t_vals64, srcc, sc, rc);
-    check_gather<T>(d.t_rowptr[j], d.t_rowptr[j + 1], d.t_cols, d.t_vals64, srca, sa, ra);
-    const double Cj = d.C[j], iCj = d.invC[j], lj = d.l64[j], uj = d.u64[j];
+  for (int q = 0; q < kNC1; ++q) acc[q] = 0.0;
+  unsigned long long h = 0ULL;
+  const T* yc = F.Y[cur] + k;
+  const T* ya = F.Y[2] + k;
+  const T* Xc = F.X[cur] + k;
+  T* Xa = F.X[2] + k;
+  auto src = [&](int i, T(&g)[2]) {
+    g[0] = g[1] = T(0);
+    if (on) {
+      const size_t o = size_t(i) * kFK;
+      g[0] = yc[o];
+      g[1] = ya[o];
+      if (avg) g[1] = blend(g[1], g[0], w1, w);
+    }
+  };
+  for (int j = gw / halves; j < d.n; j += nw / halves) {
+    double s[2];
+    T ref[2];
+    check_gather<T>(d.t_rowptr[j], d.t_rowptr[j + 1], d.t_cols, d.t_vals64, src, s, ref);
+    if (!on) continue;
+    const double iCj = d.invC[j], lj = d.l64[j], uj = d.u64[j];
     const T ljT = d.l[j], ujT = d.u[j];
-    const unsigned long long lob = F.lo_bits[j], upb = F.up_bits[j];
     const FanCostCol<double> cc{F.cc64[3 * size_t(j)], F.cc64[3 * size_t(j) + 1], F.cc64[3 * size_t(j) + 2]};
+    const size_t o = size_t(j) * kFK;
+    const T x = Xc[o];
+    // the average of points in [l, u] can leave it by a rounding: it is kept in the
+    // box the iterates are clamped to, so that the point a check evaluates is the
+    // one an objective finishing with it keeps (and returns)
+    const T x0 = Xa[o];
+    T xav = x0;
+    if (avg) xav = blend(xav, x, w1, w);
+    xav = clampv<T>(xav, ljT, ujT);
+    if (xav != x0) Xa[o] = xav;
+    F.ATY[0][o + k] = ref[0];
+    F.ATY[1][o + k] = ref[1];
+    const double cs = cc.at(int((F.lo_bits[j] >> k) & 1ULL) - int((F.up_bits[j] >> k) & 1ULL));
+    const double xl = to_f64(F.XLR[o + k]);
+    const double xs[2] = {to_f64(x), to_f64(xav)};
+    const bool boxed = above_neg_inf(lj) && below_pos_inf(uj);  // then r - lambda = 0 exactly
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      if (!on[q]) continue;
-      const int k = lane + 32 * q;
-      const size_t o = size_t(j) * kFK + k;
-      const T x = Xc[o];
-      // the average of points in [l, u] can leave it by a rounding: it is kept in the
-      // box the iterates are clamped to, so that the point a check evaluates is the
-      // one an objective finishing with it keeps (and returns)
-      const T x0 = Xa[o];
-      T xav = x0;
-      if (fl[q] & kSlotAvg) xav = blend(xav, x, w1[q], w[q]);
-      xav = clampv<T>(xav, ljT, ujT);
-      if (xav != x0) Xa[o] = xav;
-      F.ATY[0][o] = rc[q];
-      F.ATY[1][o] = ra[q];
-      const double cs = cc.at(int((lob >> k) & 1ULL) - int((upb >> k) & 1ULL));
-      const double xl = to_f64(F.XLR[o]);
-      const double xs[2] = {to_f64(x), to_f64(xav)};
-      const double ss[2] = {sc[q], sa[q]};
-      const bool boxed = above_neg_inf(lj) && below_pos_inf(uj);  // then r - lambda = 0 exactly
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const double r = cs - ss[c];
-        const double lam = rc_proj(r, lj, uj);
-        double* a = acc + q * kNC1 + 5 * c;
-        if (!boxed) {
-          const double rd = r - lam;
-          a[0] += rd * rd;
-          const double rdu = rd * iCj;
-          a[1] += rdu * rdu;
-        }
-        a[2] += cs * xs[c];
-        a[3] += bound_term(lam, lj, uj);
-        const double dd = xs[c] - xl;
-        a[4] += dd * dd;
+    for (int c = 0; c < 2; ++c) {
+      const double r = cs - s[c];
+      const double lam = rc_proj(r, lj, uj);
+      double* a = acc + 5 * c;
+      if (!boxed) {
+        const double rd = r - lam;
+        a[0] += rd * rd;
+        const double rdu = rd * iCj;
+        a[1] += rdu * rdu;
       }
-      if (hs[q] && d.int_mask[j]) h[q] += round_hash(j, xs[0] * Cj);
+      a[2] += cs * xs[c];
+      a[3] += bound_term(lam, lj, uj);
+      const double dd = xs[c] - xl;
+      a[4] += dd * dd;
     }
+    if (hs && d.int_mask[j]) h += round_hash(j, xs[0] * d.C[j]);
   }
-  store_block_sums<double>(acc, kNC1, F.part_c1, sh);
-#pragma unroll
-  for (int q = 0; q < 2; ++q)
-    if (on[q] && h[q]) atomicAdd(&F.ctl[lane + 32 * q].hash_accum, h[q]);
+  store_block_sums(acc, halves, F.part_c1, sh);
+  if (on && h) atomicAdd(&F.ctl[k].hash_accum, h);
 }
 
+// Row half of a check, laid out as the column half.
 template <typename T>
-__global__ void __launch_bounds__(kFThreads) k_fcheck_rows(DevFan<T> F) {
-  __shared__ double sh[kFWarps * kNC2 * kFK];
-  const int lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(kFThreads, 3) k_fcheck_rows(DevFan<T> F) {
+  if (*F.n_done >= F.K) return;
+  __shared__ double sh[kFWarps * kNC2 * 32];
+  const int lane = threadIdx.x & 31, halves = fan_halves(F.K);
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+  const int k = lane + 32 * (gw % halves);
   const DevLP<T>& d = F.d;
   const int cur = fan_cur(F);
-  bool on[2];
-  int fl[2];
-  T w[2], w1[2];
+  const int fl = k < F.K ? F.slot[k].flags : 0;
+  const bool on = (fl & kSlotCheck) != 0, avg = (fl & kSlotAvg) != 0;
+  const T w = k < F.K ? F.slot[k].w : T(0), w1 = k < F.K ? F.slot[k].w1 : T(1);
+  double acc[kNC2];
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int k = lane + 32 * q;
-    fl[q] = k < F.K ? F.slot[k].flags : 0;
-    on[q] = (fl[q] & kSlotCheck) != 0;
-    w[q] = k < F.K ? F.slot[k].w : T(0);
-    w1[q] = k < F.K ? F.slot[k].w1 : T(1);
-  }
-  double acc[2 * kNC2];
-#pragma unroll
-  for (int q = 0; q < 2 * kNC2; ++q) acc[q] = 0.0;
-  const T* xc = F.X[cur];
-  const T* xa = F.X[2];
-  T* Yc = F.Y[cur];
-  T* Ya = F.Y[2];
-  for (int i = gw; i < d.m; i += nw) {
-    double sc[2], sa[2];
-    T rc[2], ra[2];
-    auto srcc = [&](int j, T(&g)[2]) {
-#pragma unroll
-      for (int q = 0; q < 2; ++q) g[q] = on[q] ? xc[size_t(j) * kFK + lane + 32 * q] : T(0);
-    };
-    auto srca = [&](int j, T(&g)[2]) {
-#pragma unroll
-      for (int q = 0; q < 2; ++q) g[q] = on[q] ? xa[size_t(j) * kFK + lane + 32 * q] : T(0);
-    };
-    check_gather<T>(d.a_rowptr[i], d.a_rowptr[i + 1], d.a_cols, d.a_vals64, srcc, sc, rc);
-    check_gather<T>(d.a_rowptr[i], d.a_rowptr[i + 1], d.a_cols, d.a_vals64, srca, sa, ra);
+  for (int q = 0; q < kNC2; ++q) acc[q] = 0.0;
+  const T* xc = F.X[cur] + k;
+  const T* xa = F.X[2] + k;
+  const T* Yc = F.Y[cur] + k;
+  T* Ya = F.Y[2] + k;
+  auto src = [&](int j, T(&g)[2]) {
+    g[0] = g[1] = T(0);
+    if (on) {
+      g[0] = xc[size_t(j) * kFK];
+      g[1] = xa[size_t(j) * kFK];
+    }
+  };
+  for (int i = gw / halves; i < d.m; i += nw / halves) {
+    double s[2];
+    T ref[2];
+    check_gather<T>(d.a_rowptr[i], d.a_rowptr[i + 1], d.a_cols, d.a_vals64, src, s, ref);
+    if (!on) continue;
     const double iRi = d.invR[i], lo = d.lo64[i], hi = d.hi64[i];
+    const size_t o = size_t(i) * kFK;
+    const T y = Yc[o];
+    T yav = Ya[o];
+    if (avg) {
+      yav = blend(yav, y, w1, w);
+      Ya[o] = yav;
+    }
+    F.AX[cur][o + k] = ref[0];
+    F.AX[2][o + k] = ref[1];
+    const double yl = to_f64(F.YLR[o + k]);
+    const double ys[2] = {to_f64(y), to_f64(yav)};
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      if (!on[q]) continue;
-      const int k = lane + 32 * q;
-      const size_t o = size_t(i) * kFK + k;
-      const T y = Yc[o];
-      T yav = Ya[o];
-      if (fl[q] & kSlotAvg) {
-        yav = blend(yav, y, w1[q], w[q]);
-        Ya[o] = yav;
-      }
-      F.AX[cur][o] = rc[q];
-      F.AX[2][o] = ra[q];
-      const double yl = to_f64(F.YLR[o]);
-      const double ys[2] = {to_f64(y), to_f64(yav)};
-      const double ss[2] = {sc[q], sa[q]};
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const double rps = ss[c] - clampv<double>(ss[c], lo, hi);
-        double* a = acc + q * kNC2 + 4 * c;
-        a[0] += rps * rps;
-        const double rp = rps * iRi;
-        a[1] += rp * rp;
-        a[2] += bound_term(ys[c], lo, hi);
-        const double dd = ys[c] - yl;
-        a[3] += dd * dd;
-      }
+    for (int c = 0; c < 2; ++c) {
+      const double rps = s[c] - clampv<double>(s[c], lo, hi);
+      double* a = acc + 4 * c;
+      a[0] += rps * rps;
+      const double rp = rps * iRi;
+      a[1] += rp * rp;
+      a[2] += bound_term(ys[c], lo, hi);
+      const double dd = ys[c] - yl;
+      a[3] += dd * dd;
     }
   }
-  store_block_sums<double>(acc, kNC2, F.part_c2, sh);
+  store_block_sums(acc, halves, F.part_c2, sh);
 }
 
-// One warp per objective: check sums in a fixed order, then check_control.  An
+// A block per objective: check sums in a fixed order (a warp per sum), then check_control.  An
 // objective that restarts to its average or finishes with it (the single-LP path
 // swaps its pool roles) gets rst[k] = 1 instead, and k_fcopy_rst copies the
 // average into the current pool.  Block 0 refills the step-size factor table
 // shared by the objectives still running.
+constexpr int kFCheckThreads = (kNC1 + kNC2) * 32;
 template <typename T>
-__global__ void __launch_bounds__(kFThreads) k_fcheck_control(DevFan<T> F) {
+__global__ void __launch_bounds__(kFCheckThreads) k_fcheck_control(DevFan<T> F) {
+  if (*F.n_done >= F.K) return;
   FanState* st = F.state;
   const long long k0 = *F.kglob;
   constexpr bool f32 = sizeof(T) == 4;
-  // the step-size factors of attempts k0 + 1 .. k0 + n_check (entry i: attempt
-  // k0 + 1 + i), shared by the objectives still running: FP64 for the FP64 decision,
-  // FP32 (after the FP64 entries) for the FP32-mixed one
-  if (blockIdx.x == 0)
-    for (int i = threadIdx.x; i < F.d.n_check; i += blockDim.x) {
+  const int k = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  // the last block: the step-size factors of attempts k0 + 1 .. k0 + n_check (entry i:
+  // attempt k0 + 1 + i), shared by the objectives still running: FP64 for the FP64
+  // decision, FP32 (after the FP64 entries) for the FP32-mixed one
+  if (k == F.K) {
+    for (int q = threadIdx.x; q < 2 * F.d.n_check; q += blockDim.x) {
       if (f32) {
-        float* facf = reinterpret_cast<float*>(F.d.step_fac + 2 * F.d.n_check);
-        const float kk = float(k0 + 1 + i + 1);
-        facf[2 * i] = 1.0f - powf(kk, -float(F.exp_red));
-        facf[2 * i + 1] = 1.0f + powf(kk, -float(F.exp_grow));
+        const float kk = float(k0 + 1 + (q >> 1) + 1);
+        reinterpret_cast<float*>(F.d.step_fac + 2 * F.d.n_check)[q] =
+            (q & 1) ? 1.0f + powf(kk, -float(F.exp_grow)) : 1.0f - powf(kk, -float(F.exp_red));
       } else {
-        const double kk = double(k0 + 1 + i + 1);
-        F.d.step_fac[2 * i] = 1.0 - pow(kk, -F.exp_red);
-        F.d.step_fac[2 * i + 1] = 1.0 + pow(kk, -F.exp_grow);
+        const double kk = double(k0 + 1 + (q >> 1) + 1);
+        F.d.step_fac[q] = (q & 1) ? 1.0 + pow(kk, -F.exp_grow) : 1.0 - pow(kk, -F.exp_red);
       }
     }
-  const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (k >= F.K) return;
-  if (!(F.slot[k].flags & kSlotCheck)) {
-    if (lane == 0) st->rst[k] = 0;
     return;
   }
-  double r[kNC1 + kNC2];
-#pragma unroll
-  for (int s = 0; s < kNC1 + kNC2; ++s) r[s] = 0.0;
-  for (int b = lane; b < F.grid_c1; b += 32)
-#pragma unroll
-    for (int s = 0; s < kNC1; ++s) r[s] += F.part_c1[(b * kNC1 + s) * kFK + k];
-  for (int b = lane; b < F.grid_c2; b += 32)
-#pragma unroll
-    for (int s = 0; s < kNC2; ++s) r[kNC1 + s] += F.part_c2[(b * kNC2 + s) * kFK + k];
-#pragma unroll
-  for (int s = 0; s < kNC1 + kNC2; ++s) r[s] = fwarp_sum(r[s]);
+  if (!(F.slot[k].flags & kSlotCheck)) {
+    if (threadIdx.x == 0) st->rst[k] = 0;
+    return;
+  }
+  __shared__ double red[kNC1 + kNC2];
+  {
+    const bool col = w < kNC1;
+    const int s = col ? w : w - kNC1, N = col ? kNC1 : kNC2;
+    const double v = warp_sum(chain_sum(col ? F.part_c1 : F.part_c2, N * kFK, s * kFK + k, lane,
+                                        col ? F.grid_c1 : F.grid_c2, 32));
+    if (lane == 0) red[w] = v;
+  }
+  __syncthreads();
+  if (w != 0) return;
+  Control* c = &F.ctl[k];
+  const int ix0 = c->ix_cur, ia0 = c->ia_cur;
+  __syncwarp();
   if (lane == 0) {
-    Control* c = &F.ctl[k];
-    const int ix0 = c->ix_cur, ia0 = c->ia_cur;
     c->k_fac = k0;
     if (f32) {
       sync_step_state(c);  // eta and the weight sum from their FP32 copies
@@ -1031,7 +1010,10 @@ __global__ void __launch_bounds__(kFThreads) k_fcheck_control(DevFan<T> F) {
       c->fr_f = 1.0f - powf(kk, -float(F.exp_red));
       c->fg_f = 1.0f + powf(kk, -float(F.exp_grow));
     }
-    check_control(c, r, nullptr, 0);
+  }
+  __syncwarp();
+  check_control_warp(c, red, nullptr, 0);
+  if (lane == 0) {
     st->rst[k] = 0;
     if (c->ix_cur != ix0) {  // to the average: copy instead of swapping roles
       st->rst[k] = 1;
@@ -1052,6 +1034,8 @@ __global__ void __launch_bounds__(kFThreads) k_fcheck_control(DevFan<T> F) {
 // per (row, flagged objective) pair; nothing to do unless a flag is set.
 template <typename T, bool RST>
 __global__ void __launch_bounds__(kFThreads) k_fcopy(DevFan<T> F) {
+  // every objective finished: no attempt was made, the flags are an earlier one's
+  if (!RST && *F.n_done >= F.K) return;
   const FanState* st = F.state;
   const unsigned char* flag = RST ? st->rst : st->rej;
   // the flagged objectives, ascending
@@ -1230,14 +1214,13 @@ cudaError_t launch_fan_init(const DevFan<T>& F, double tol, long long iter_limit
 // step control, 7 copies after the check control
 template <typename T>
 cudaError_t launch_fan_part(const DevFan<T>& F, int part, cudaStream_t st) {
-  const int ctl_grid = (F.K * 32 + kFThreads - 1) / kFThreads;
   switch (part) {
     case 0: return launch_spmm<T>(F, 0, st);
     case 1: return launch_spmm<T>(F, 1, st);
-    case 2: k_fstep_control<T><<<ctl_grid, kFThreads, 0, st>>>(F); break;
+    case 2: k_fstep_control<T><<<F.K, kFStepThreads, 0, st>>>(F); break;
     case 3: k_fcheck_cols<T><<<F.grid_c1, kFThreads, 0, st>>>(F); break;
     case 4: k_fcheck_rows<T><<<F.grid_c2, kFThreads, 0, st>>>(F); break;
-    case 5: k_fcheck_control<T><<<ctl_grid, kFThreads, 0, st>>>(F); break;
+    case 5: k_fcheck_control<T><<<F.K + 1, kFCheckThreads, 0, st>>>(F); break;
     case 6: k_fcopy<T, false><<<F.grid_copy, kFThreads, 0, st>>>(F); break;
     default: k_fcopy<T, true><<<F.grid_copy, kFThreads, 0, st>>>(F); break;
   }
@@ -1297,8 +1280,9 @@ void fan_grids(DevFan<T>& F) {
   const int rpw_d = 32 * fan_shape_vec(F.shape_d) / fan_shape_chunk(F.shape_d);
   F.grid_p = grid(fan_spmm_kernel<T>(0, F.shape_p), (F.d.n + rpw_p - 1) / rpw_p);
   F.grid_d = grid(fan_spmm_kernel<T>(1, F.shape_d), (F.d.m + rpw_d - 1) / rpw_d);
-  F.grid_c1 = grid((const void*)k_fcheck_cols<T>, F.d.n);
-  F.grid_c2 = grid((const void*)k_fcheck_rows<T>, F.d.m);
+  const long long halves = F.K > 32 ? 2 : 1;
+  F.grid_c1 = grid((const void*)k_fcheck_cols<T>, halves * F.d.n);
+  F.grid_c2 = grid((const void*)k_fcheck_rows<T>, halves * F.d.m);
   F.grid_copy = grid((const void*)k_fcopy<T, false>, F.d.n > F.d.m ? F.d.n : F.d.m);
 }
 

@@ -2161,22 +2161,6 @@ __device__ __forceinline__ unsigned int atom_add_release_gpu(unsigned int* p, un
 }
 __device__ __forceinline__ void fence_acquire_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
-// a control block into a warp's shared copy (L2 loads) and back, word by word
-__device__ __forceinline__ void ctl_in(Control* dst, const Control* src) {
-  static_assert(sizeof(Control) % 4 == 0, "word copy");
-  const int lane = threadIdx.x & 31;
-  for (int i = lane; i < int(sizeof(Control) / 4); i += 32)
-    reinterpret_cast<int*>(dst)[i] = __ldcg(reinterpret_cast<const int*>(src) + i);
-  __syncwarp();
-}
-__device__ __forceinline__ void ctl_out(Control* dst, const Control* src) {
-  __syncwarp();
-  const int lane = threadIdx.x & 31;
-  for (int i = lane; i < int(sizeof(Control) / 4); i += 32)
-    reinterpret_cast<int*>(dst)[i] = reinterpret_cast<const int*>(src)[i];
-  __syncwarp();
-}
-
 // the decision of one LP on its shared control copy: out of line, so that its
 // registers do not count against the matrix phases of the persistent kernel
 template <typename T>
@@ -2288,21 +2272,6 @@ struct BDualEpi : DualEpi<T, Coh> {
   }
 };
 
-// One lane's chain of per-tile values part[t * stride + off], t = beg, beg + step, ... <
-// end, added in that order; eight loads in flight.
-__device__ __forceinline__ double lp_chain_sum(const double* part, int stride, int off, int beg, int end, int step) {
-  double v = 0.0;
-  for (int t = beg; t < end; t += 8 * step) {
-    double x[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = t + u * step < end ? __ldcg(part + size_t(t + u * step) * stride + off) : 0.0;
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (t + u * step < end) v += x[u];
-  }
-  return v;
-}
-
 // A block per LP: its tiles' sums in lp_tile_sum's order, then the step decision (the
 // launch-per-phase path).  Warp 4 k + u takes the fourth u of sum k's running sums, so
 // the largest LP's chain is a twelfth of one warp's work and its loads come eight at a
@@ -2321,7 +2290,7 @@ __global__ void __launch_bounds__(kBStepThreads) k_bstep_control(DevBatch<T> B) 
   {
     const int beg = __ldg((k == 0 ? B.t_tile_beg : B.a_tile_beg) + b);
     const int end = __ldg((k == 0 ? B.t_tile_beg : B.a_tile_beg) + b + 1);
-    sh[w][lane] = lp_chain_sum(k == 0 ? B.tp_p : B.tp_d, k == 0 ? 1 : 2, k == 2 ? 1 : 0, beg + lane + 32 * u, end, 128);
+    sh[w][lane] = chain_sum(k == 0 ? B.tp_p : B.tp_d, k == 0 ? 1 : 2, k == 2 ? 1 : 0, beg + lane + 32 * u, end, 128);
   }
   __syncthreads();
   if (w < 3) {
@@ -2529,7 +2498,7 @@ __global__ void __launch_bounds__(kBCheckThreads) k_bcheck_control(DevBatch<T> B
   {
     const bool col = w < kNC1;
     const int beg = __ldg((col ? B.t_tile_beg : B.a_tile_beg) + b), end = __ldg((col ? B.t_tile_beg : B.a_tile_beg) + b + 1);
-    const double v = warp_sum(lp_chain_sum(col ? B.tp_c1 : B.tp_c2, col ? kNC1 : kNC2, col ? w : w - kNC1, beg + lane,
+    const double v = warp_sum(chain_sum(col ? B.tp_c1 : B.tp_c2, col ? kNC1 : kNC2, col ? w : w - kNC1, beg + lane,
                                            end, 32));
     if (lane == 0) red[w] = v;
   }
@@ -2582,6 +2551,13 @@ __global__ void k_bget_x(DevBatch<T> B, int b, int col0, int count, double* out)
   const T* x = B.d.X[B.ctl[b].ix_cur];
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < count; j += gridDim.x * blockDim.x)
     out[j] = double(x[col0 + j]) * B.d.C[col0 + j];
+}
+
+template <typename T>
+__global__ void k_bget_y(DevBatch<T> B, int b, int row0, int count, double* out) {
+  const T* y = B.d.Y[B.ctl[b].ix_cur];
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x)
+    out[i] = double(y[row0 + i]) * B.d.R[row0 + i];
 }
 
 template <typename T>
@@ -3182,6 +3158,11 @@ cudaError_t launch_batch_get_x(const DevBatch<T>& B, int b, int col0, int count,
   return cudaGetLastError();
 }
 template <typename T>
+cudaError_t launch_batch_get_y(const DevBatch<T>& B, int b, int row0, int count, double* out, cudaStream_t st) {
+  k_bget_y<T><<<ew_grid(count), kThreads, 0, st>>>(B, b, row0, count, out);
+  return cudaGetLastError();
+}
+template <typename T>
 cudaError_t launch_batch_init_point(const DevBatch<T>& B, cudaStream_t st) {
   k_binit_point<T><<<ew_grid(B.d.m > B.d.n ? B.d.m : B.d.n), kThreads, 0, st>>>(B);
   return cudaGetLastError();
@@ -3252,6 +3233,7 @@ void batch_grids(DevBatch<T>& B) {
   template cudaError_t launch_batch_slot<T>(const DevBatch<T>&, cudaStream_t);                         \
   template cudaError_t launch_batch_check<T>(const DevBatch<T>&, cudaStream_t);                        \
   template cudaError_t launch_batch_part<T>(const DevBatch<T>&, int, cudaStream_t);                    \
+  template cudaError_t launch_batch_get_y<T>(const DevBatch<T>&, int, int, int, double*, cudaStream_t); \
   template cudaError_t launch_batch_get_x<T>(const DevBatch<T>&, int, int, int, double*, cudaStream_t); \
   template cudaError_t launch_batch_init_point<T>(const DevBatch<T>&, cudaStream_t);                   \
   template void batch_grids<T>(DevBatch<T>&);                                                            \
