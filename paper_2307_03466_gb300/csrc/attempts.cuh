@@ -170,7 +170,7 @@ __device__ __forceinline__ void res_load(const ResSide<T>& S, int i, ResTile& R,
   }
   const int2 ta = __ldg(S.tiles + t), tb = __ldg(S.tiles + t + 1);
   const int nr = tb.x - ta.x, n = tb.y - ta.y;
-  R.lsh = nr > 1 ? (nr >= 32 ? 0 : __clz(nr - 1) - 27) : 5;
+  R.lsh = row_lanes_log2(nr);
   const int rl = lane >> R.lsh, sub = lane & ((1 << R.lsh) - 1);
   if (rl < nr) {
     R.q0 = __ldg(S.rowptr + ta.x + rl) - ta.y + sub;

@@ -33,6 +33,11 @@ __device__ __forceinline__ int row_lanes(int nr) {
   const int l = 32 / (nr > 0 ? nr : 1);
   return 1 << (31 - __clz(l));
 }
+// Its base-2 logarithm by shifts: an integer division by a run-time value is some twenty
+// instructions, and two more divisions map a lane to its row.  (spmv_tiles keeps the
+// divisions: its L = 1 tiles branch past them, and the shift form was 3 to 7% slower on
+// the multicommodity-flow workload.)
+__device__ __forceinline__ int row_lanes_log2(int nr) { return nr >= 32 ? 0 : nr > 1 ? __clz(nr - 1) - 27 : 5; }
 
 // The tiles of a warp: tile t goes to block t mod G and, within the block, to warp
 // (t div G) mod 8, so every block holds the same number of tiles (within one) and
@@ -241,17 +246,24 @@ struct NoPro {
   __device__ __forceinline__ bool operator()() const { return true; }
 };
 
-// Check form of the gather over FP32 iterates: the multi-row path stores each FP64
-// value and the gathered FP32 entries, and every row sum is a chain of FP64 fused
+// entries that a lane gathers ahead of its sum where it gathers the entries it sums
+constexpr int kOwnAhead = 8;
+
+// Check form of the gather over FP32 iterates: every row sum is a chain of FP64 fused
 // multiply-adds of a value and an exactly converted entry, in CSR order (one FP64
 // instruction per nonzero and vector instead of a conversion, a product and a sum).
-// smw holds kSmemPerWarp doubles, then NV * kSmemPerWarp floats.
+// The multi-row path stages the tile's indices and values in shared memory, and the lane
+// that sums an entry gathers it, kOwnAhead entries at a time: the gathered entries need no
+// way through shared memory, and neighbouring rows with neighbouring columns (network and
+// multi-period models) gather whole lines.  (packing/covering 200k x 500k: column check
+// 127 -> 99 us, row check 162 -> 141.)
+// smw holds kSmemPerWarp doubles, then kSmemPerWarp ints.
 template <int NV, typename Gather, typename Epi>
 __device__ __forceinline__ void spmv_tiles_fma(const int2* __restrict__ tiles, int ntiles,
                                                const int* __restrict__ rowptr, const int* __restrict__ cols,
                                                const double* __restrict__ vals, Gather& gat, Epi& epi,
                                                double* __restrict__ smw) {
-  float* __restrict__ sg = reinterpret_cast<float*>(smw + kSmemPerWarp);
+  int* __restrict__ sc = reinterpret_cast<int*>(smw + kSmemPerWarp);
   const int lane = threadIdx.x & 31;
   const WarpTiles wt = warp_tiles(ntiles);
   for (int t = wt.first; t < wt.end; t += wt.step) {
@@ -283,7 +295,7 @@ __device__ __forceinline__ void spmv_tiles_fma(const int2* __restrict__ tiles, i
       for (int k = 0; k < NV; ++k) s[k] = warp_sum(s[k]);
       if (lane == 0) epi.finish(r0, s, pre);
     } else {
-      const int L = row_lanes(r1 - r0), rl = lane / L, sub = lane - rl * L;
+      const int sh = row_lanes_log2(r1 - r0), L = 1 << sh, rl = lane >> sh, sub = lane & (L - 1);
       const bool mine = rl < r1 - r0, lead = mine && sub == 0;
       const int row = r0 + rl;
       int q0 = 0, q1 = 0;
@@ -310,12 +322,9 @@ __device__ __forceinline__ void spmv_tiles_fma(const int2* __restrict__ tiles, i
         for (int e = 0; e < 4; ++e) {
           const int q = p + e;
           if (q >= p0 && q < p1) {
-            float g[NV];
-            gat(c[it][e], g);
             const int o = skew(q - p0);
             smw[o] = v[it][e];
-#pragma unroll
-            for (int k = 0; k < NV; ++k) sg[k * kSmemPerWarp + o] = g[k];
+            sc[o] = c[it][e];
           }
         }
       }
@@ -324,11 +333,18 @@ __device__ __forceinline__ void spmv_tiles_fma(const int2* __restrict__ tiles, i
 #pragma unroll
       for (int k = 0; k < NV; ++k) s[k] = 0.0;
       if (mine) {
-        for (int q = q0 + sub; q < q1; q += L) {
-          const int o = skew(q);
-          const double a = smw[o];
+        for (int q = q0 + sub; q < q1; q += kOwnAhead * L) {
+          float g[kOwnAhead][NV];
 #pragma unroll
-          for (int k = 0; k < NV; ++k) s[k] = __fma_rn(a, to_f64(sg[k * kSmemPerWarp + o]), s[k]);
+          for (int u = 0; u < kOwnAhead; ++u)
+            if (q + u * L < q1) gat(sc[skew(q + u * L)], g[u]);
+#pragma unroll
+          for (int u = 0; u < kOwnAhead; ++u)
+            if (q + u * L < q1) {
+              const double a = smw[skew(q + u * L)];
+#pragma unroll
+              for (int k = 0; k < NV; ++k) s[k] = __fma_rn(a, to_f64(g[u][k]), s[k]);
+            }
         }
       }
       for (int o = L >> 1; o > 0; o >>= 1)
@@ -427,10 +443,10 @@ __device__ __forceinline__ void tiles_rows(const int2* __restrict__ tiles, int n
   const WarpTiles wt = warp_tiles(ntiles);
   for (int t = wt.first; t < wt.end; t += wt.step) {
     const int2 ta = __ldg(tiles + t), tb = __ldg(tiles + t + 1);
-    const int nr = tb.x - ta.x, L = row_lanes(nr);
-    if (L > 1) {
-      if (lane % L == 0 && lane / L < nr) {
-        const int row = ta.x + lane / L;
+    const int nr = tb.x - ta.x, sh = row_lanes_log2(nr);
+    if (sh > 0) {
+      if ((lane & ((1 << sh) - 1)) == 0 && lane >> sh < nr) {
+        const int row = ta.x + (lane >> sh);
         const T s[1] = {src[row]};
         epi.finish(row, s, epi.load(row));
       }
@@ -538,8 +554,8 @@ __device__ __forceinline__ void spmv_tiles_async(const int2* __restrict__ tiles,
       long_row_sum<1, true>(p0, p1, cols, vals, gat, s);
       if (lane == 0) epi.finish(r0, s, pre);
     } else {
-      const int nr = r1 - r0, L = row_lanes(nr), sub = L > 1 ? lane % L : 0;
-      const int rl = L > 1 ? lane / L : lane;
+      const int nr = r1 - r0, sh = row_lanes_log2(nr), L = 1 << sh, sub = lane & (L - 1);
+      const int rl = lane >> sh;
       int q0 = 0, q1 = 0;
       typename Epi::Pre pre{};
       if (rl < nr) {
@@ -1019,14 +1035,14 @@ __device__ bool staged_tiles(const int2* __restrict__ tiles, int ntiles, const i
       T* sval = reinterpret_cast<T*>(st + S::kValsOff);
       const int* srp = reinterpret_cast<const int*>(st + S::kRpOff);
       const T* svec = reinterpret_cast<const T*>(st + S::kVecOff);
-      // rows as in spmv_tiles on wide tiles: slot j of a lane is row lane / L (rows
+      // rows as in spmv_tiles on wide tiles: slot j of a lane is row lane >> sh (rows
       // split over L lanes) or row lane + 32 j
-      const int nr = b.r1 - b.r0, L = row_lanes(nr), sub = L > 1 ? lane % L : 0;
+      const int nr = b.r1 - b.r0, sh = row_lanes_log2(nr), L = 1 << sh, sub = lane & (L - 1);
       int q0[kWideRPL], q1[kWideRPL];
       typename Epi::Pre pre[kWideRPL];
 #pragma unroll
       for (int j = 0; j < kWideRPL; ++j) {
-        const int rl = L > 1 ? (j == 0 ? lane / L : nr) : lane + 32 * j;
+        const int rl = sh > 0 ? (j == 0 ? lane >> sh : nr) : lane + 32 * j;
         q0[j] = q1[j] = 0;
         pre[j] = typename Epi::Pre{};
         if (rl < nr) {
@@ -1052,7 +1068,7 @@ __device__ bool staged_tiles(const int2* __restrict__ tiles, int ntiles, const i
       __syncwarp();
 #pragma unroll
       for (int j = 0; j < kWideRPL; ++j) {
-        const int rl = L > 1 ? (j == 0 ? lane / L : nr) : lane + 32 * j;
+        const int rl = sh > 0 ? (j == 0 ? lane >> sh : nr) : lane + 32 * j;
         T acc = T(0);
         if (rl < nr && !skip_gather)
           for (int q = q0[j] + sub; q < q1[j]; q += L) acc += sval[off + q];
