@@ -306,6 +306,10 @@ cudaError_t launch_precondition(const DevSetup& s, int ruiz_iters, bool pock_cha
 // a~ = diag(R) A diag(C) in both CSR copies (and their FP32 shadows)
 cudaError_t launch_scale_values(const DevSetup& s, cudaStream_t st);
 cudaError_t fill_f64(double* p, long long count, double v, cudaStream_t st);
+// *bad = 1 when the arrays are malformed (scylla_lp_create); bad is cleared by the caller
+cudaError_t check_malformed(int m, int n, int nnz, const int* rowptr, const int* cols, const double* vals,
+                            const double* c, const double* lo, const double* hi, const double* l, const double* u,
+                            const uint8_t* is_int, int* bad, cudaStream_t st);
 // l64 = l / C, u64 = u / C (and the FP32 shadows when given) over n columns
 cudaError_t scale_col_bounds(long long n, const double* l, const double* u, const double* C, double* l64,
                              double* u64, float* l32, float* u32, cudaStream_t st);

@@ -272,8 +272,9 @@ void scylla_lp::ensure_columns() const {
 }
 
 // --------------------------------------------------------------- validation ---
-int scylla::validate_lp(const scylla_csr* A, const double* c, const double* lo, const double* hi, const double* l,
-                    const double* u, const uint8_t* is_int) {
+// what the sizes and the row pointers must satisfy before the other arrays can be read
+static int validate_structure(const scylla_csr* A, const double* c, const double* lo, const double* hi,
+                              const double* l, const double* u, const uint8_t* is_int) {
   if (!A || !c || !lo || !hi || !l || !u || !is_int) FAIL(SCYLLA_ERR_INVALID_ARG, "null argument");
   if (A->m < 0 || A->n < 1 || A->nnz < 0) FAIL(SCYLLA_ERR_INVALID_ARG, "need m >= 0, n >= 1, nnz >= 0");
   const int64_t lim = (int64_t(1) << 31) - 64;
@@ -283,6 +284,13 @@ int scylla::validate_lp(const scylla_csr* A, const double* c, const double* lo, 
   if (A->rowptr[0] != 0 || A->rowptr[A->m] != A->nnz) FAIL(SCYLLA_ERR_INVALID_ARG, "rowptr[0] != 0 or rowptr[m] != nnz");
   for (int64_t i = 0; i < A->m; ++i)
     if (A->rowptr[i + 1] < A->rowptr[i]) FAIL(SCYLLA_ERR_INVALID_ARG, "rowptr not non-decreasing at row " + std::to_string(i));
+  return SCYLLA_OK;
+}
+
+int scylla::validate_lp(const scylla_csr* A, const double* c, const double* lo, const double* hi, const double* l,
+                    const double* u, const uint8_t* is_int) {
+  const int rs = validate_structure(A, c, lo, hi, l, u, is_int);
+  if (rs != SCYLLA_OK) return rs;
   // rows in parallel slices; the first failing row is reported
   {
     const int64_t mm = A->m;
@@ -361,7 +369,7 @@ int scylla::validate_lp(const scylla_csr* A, const double* c, const double* lo, 
 // ------------------------------------------------------------------ create ---
 static int create_impl(const scylla_csr* A, const double* c, const double* lo, const double* hi, const double* l,
                        const double* u, const uint8_t* is_int, const scylla_params* pin, void* cuda_stream,
-                       scylla_lp* lp) {
+                       scylla_lp* lp, bool check_on_device) {
   lp->p = *pin;
   if (lp->p.n_check < 1) FAIL(SCYLLA_ERR_INVALID_ARG, "n_check must be >= 1");
   if (lp->p.trace_capacity < 0) FAIL(SCYLLA_ERR_INVALID_ARG, "trace_capacity must be >= 0");
@@ -386,10 +394,9 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
   CK(cudaEventCreate(&lp->ev0));
   CK(cudaEventCreate(&lp->ev1));
 
-  // ---- the original MIP: ||c||, the integer count and the general integers that
-  // get auxiliary columns, in one pass over the caller's arrays in a number of
-  // chunks fixed by n (so ||c|| does not depend on the host's thread count).  The
-  // host copies of the vectors are fetched from the device on first use.
+  // ---- the original MIP: the integer count and the general integers that get auxiliary
+  // columns (||c|| is summed below, while the device preconditions).  The host copies of
+  // the vectors are fetched from the device on first use.
   const int64_t m0 = A->m, n0 = A->n, nnz0 = A->nnz;
   lp->m0 = m0;
   lp->n0 = n0;
@@ -397,32 +404,28 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
   // the l2 distance needs no auxiliary columns
   const bool aux_on = lp->p.aux_general_integers != 0 && lp->p.distance == 1;
   {
+    int64_t k = 0;
+    for (int64_t j = 0; j < n0; ++j) k += is_int[j] != 0;
+    lp->n_int = k;
+    lp->gen_int.clear();
+    if (aux_on && k > 0)
+      for (int64_t j = 0; j < n0; ++j)
+        if (is_int[j] && u[j] - l[j] != 1.0) lp->gen_int.push_back(int32_t(j));
+  }
+  // ||c||: in chunks fixed by n, each in order, so that it does not depend on the host's
+  // thread count
+  auto c_norm = [&] {
     const int chunks = int(std::max<int64_t>(1, std::min<int64_t>(64, n0 / 65536)));
     std::vector<double> c2(size_t(chunks), 0.0);
-    std::vector<int64_t> nint(size_t(chunks), 0);
-    std::vector<std::vector<int32_t>> gen(static_cast<size_t>(chunks));
     fork_join(chunks, [&](int t) {
       double s2 = 0.0;
-      int64_t k = 0;
-      for (int64_t j = n0 * t / chunks; j < n0 * (t + 1) / chunks; ++j) {
-        s2 += c[j] * c[j];
-        if (!is_int[j]) continue;
-        ++k;
-        if (aux_on && u[j] - l[j] != 1.0) gen[size_t(t)].push_back(int32_t(j));
-      }
+      for (int64_t j = n0 * t / chunks; j < n0 * (t + 1) / chunks; ++j) s2 += c[j] * c[j];
       c2[size_t(t)] = s2;
-      nint[size_t(t)] = k;
     });
     double s2 = 0.0;
-    lp->n_int = 0;
-    lp->gen_int.clear();
-    for (int t = 0; t < chunks; ++t) {
-      s2 += c2[size_t(t)];
-      lp->n_int += nint[size_t(t)];
-      lp->gen_int.insert(lp->gen_int.end(), gen[size_t(t)].begin(), gen[size_t(t)].end());
-    }
-    lp->c0norm = std::sqrt(s2);
-  }
+    for (int t = 0; t < chunks; ++t) s2 += c2[size_t(t)];
+    return std::sqrt(s2);
+  };
   const int64_t na = int64_t(lp->gen_int.size());
   lp->n_aux = na;
   const int64_t m = m0 + 2 * na, n = n0 + na, nnz = nnz0 + 4 * na;
@@ -499,7 +502,8 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
   // in flight: wide tiles (up to kWideRows rows, several per lane; several times the
   // bytes of a 32-row tile on short rows) and 80 registers, which keep more loads in
   // flight per warp.  prefetch = 1 .. 4 force a form.
-  std::vector<int2> atw, ttw;
+  std::vector<int2> atw;
+  bool later_w = false;
   {
     int l2 = 0;
     CK(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, lp->device));
@@ -518,11 +522,13 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
     lp->form_rule = pf == 0 ? form : (fits ? kFormPlain : kFormWide);
     lp->tune = pf == 0 && lp->p.autotune != 0;
     auto wide_form = [](int f) { return f == kFormWide || f == kFormStaged; };
-    if (wide_form(lp->form_p) || wide_form(lp->form_d) || lp->tune) atw = build_tiles(rp, kWideRows);
+    later_w = lp->tune && lp->form_rule == kFormPlain;
+    if (wide_form(lp->form_p) || wide_form(lp->form_d) || (lp->tune && !later_w)) atw = build_tiles(rp, kWideRows);
   }
-  // wide tiles are built for the wide forms, and for the autotuner, which times both
-  const bool wide_p = lp->form_p == kFormWide || lp->form_p == kFormStaged || lp->tune;
-  const bool wide_d = lp->form_d == kFormWide || lp->form_d == kFormStaged || lp->tune;
+  // wide tiles are built for the wide forms, and for the autotuner, which times both: for
+  // an LP that stays in L2 only once it turns out that it cannot run resident
+  const bool wide_p = lp->form_p == kFormWide || lp->form_p == kFormStaged || (lp->tune && !later_w);
+  const bool wide_d = lp->form_d == kFormWide || lp->form_d == kFormStaged || (lp->tune && !later_w);
   lp->a_ntiles_w = wide_d ? int(atw.size()) - 1 : lp->a_ntiles;
   auto grid_of = [&](int side, int form, int tiles) {
     return mixed ? occupancy_grid<float>(side, form, tiles) : occupancy_grid<double>(side, form, tiles);
@@ -536,7 +542,7 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
   const int cap_c1 = grid_of(2, 0, 1 << 30);
   if (lp->tune) {
     cap_p = std::max(grid_of(0, kFormPlain, 1 << 30), grid_of(0, kFormWide, 1 << 30));
-    cap_d = std::max(grid_of(1, kFormPlain, lp->a_ntiles), grid_of(1, kFormWide, lp->a_ntiles_w));
+    cap_d = std::max(grid_of(1, kFormPlain, lp->a_ntiles), grid_of(1, kFormWide, later_w ? 1 << 30 : lp->a_ntiles_w));
     if (mixed) {
       cap_p = std::max(cap_p, grid_of(0, kFormAsync, 1 << 30));
       cap_d = std::max(cap_d, grid_of(1, kFormAsync, lp->a_ntiles));
@@ -654,6 +660,22 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
   if (wide_d) CK(cudaMemcpyAsync(lp->a_tiles_w, atw.data(), sizeof(int2) * atw.size(), cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(lp->a_vals64, va, sizeof(double) * nnz, cudaMemcpyHostToDevice, st));
   if (nnz > 0) CK(cudaMemcpyAsync(lp->a_vals0, lp->a_vals64, sizeof(double) * nnz, cudaMemcpyDeviceToDevice, st));
+  CK(cudaMemcpyAsync(lp->c_un, cP, sizeof(double) * n, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(lp->l_un, lP, sizeof(double) * n, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(lp->u_un, uP, sizeof(double) * n, cudaMemcpyHostToDevice, st));
+  if (m > 0) {
+    CK(cudaMemcpyAsync(lp->lo_un, loP, sizeof(double) * m, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(lp->hi_un, hiP, sizeof(double) * m, cudaMemcpyHostToDevice, st));
+  }
+  CK(cudaMemcpyAsync(lp->int_mask, imP, n, cudaMemcpyHostToDevice, st));
+  if (check_on_device) {
+    int* bad = reinterpret_cast<int*>(lp->red_c1);  // zero from the arena's clearing
+    CK(check_malformed(int(m0), int(n0), int(nnz0), lp->a_rowptr, lp->a_cols, lp->a_vals64, lp->c_un, lp->lo_un,
+                       lp->hi_un, lp->l_un, lp->u_un, lp->int_mask, bad, st));
+    CK(cudaMemcpyAsync(lp->h_done, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    if (lp->h_done[0] != 0) FAIL(SCYLLA_ERR_INVALID_ARG, "malformed LP");  // the host check says where
+  }
   if (host_tp) {
     CK(cudaMemcpyAsync(lp->t_rowptr, tp.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(lp->t_cols, tr.data(), sizeof(int) * nnz, cudaMemcpyHostToDevice, st));
@@ -687,14 +709,6 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
     lp->grid_c1 = grid_of(2, 0, lp->t_ntiles);
     CK(cudaStreamSynchronize(st));  // tt and ttw leave scope
   }
-  CK(cudaMemcpyAsync(lp->c_un, cP, sizeof(double) * n, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(lp->l_un, lP, sizeof(double) * n, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(lp->u_un, uP, sizeof(double) * n, cudaMemcpyHostToDevice, st));
-  if (m > 0) {
-    CK(cudaMemcpyAsync(lp->lo_un, loP, sizeof(double) * m, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(lp->hi_un, hiP, sizeof(double) * m, cudaMemcpyHostToDevice, st));
-  }
-  CK(cudaMemcpyAsync(lp->int_mask, imP, n, cudaMemcpyHostToDevice, st));
   // the original columns are the first n0 of the iterated LP's
   CK(cudaMemcpyAsync(lp->c_orig, lp->c_un, sizeof(double) * n0, cudaMemcpyDeviceToDevice, st));
   CK(cudaMemcpyAsync(lp->l_orig, lp->l_un, sizeof(double) * n0, cudaMemcpyDeviceToDevice, st));
@@ -726,6 +740,7 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
     s.R = lp->R; s.C = lp->C; s.R2 = lp->R2; s.C2 = lp->C2; s.red = lp->red; s.red_blocks = lp->red_blocks;
     CK(launch_precondition(s, lp->p.ruiz_iters, lp->p.pock_chambolle != 0, st));
     CK(launch_scale_values(s, st));
+    lp->c0norm = c_norm();
     DevVecs v{};
     v.c = lp->c_un; v.lo = lp->lo_un; v.hi = lp->hi_un; v.l = lp->l_un; v.u = lp->u_un;
     v.c64 = lp->c64; v.lo64 = lp->lo64; v.hi64 = lp->hi64; v.l64 = lp->l64; v.u64 = lp->u64;
@@ -776,6 +791,21 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
       lp->tune = false;
       if (lp->p.use_graph == 1) lp->resident = plan;
     }
+  }
+  if (lp->tune && later_w) {
+    const std::vector<int2> aw = build_tiles(rp, kWideRows), tw = build_tiles(tp, kWideRows);
+    cudaMemPool_t pool = nullptr;
+    CK(handle_pool(lp->device, &pool));
+    CK(cudaMallocFromPoolAsync(&lp->arena_w, sizeof(int2) * (aw.size() + tw.size()), pool, st));
+    lp->a_tiles_w = static_cast<int2*>(lp->arena_w);
+    lp->t_tiles_w = lp->a_tiles_w + aw.size();
+    lp->a_ntiles_w = int(aw.size()) - 1;
+    lp->t_ntiles_w = int(tw.size()) - 1;
+    CK(cudaMemcpyAsync(lp->a_tiles_w, aw.data(), sizeof(int2) * aw.size(), cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(lp->t_tiles_w, tw.data(), sizeof(int2) * tw.size(), cudaMemcpyHostToDevice, st));
+    CK(cudaStreamSynchronize(st));
+    if (mixed) fill_dev<float>(lp->d32, lp);
+    else fill_dev<double>(lp->d64, lp);
   }
   if (lp->tune) {
     const int rc = mixed ? autotune_form<float>(lp) : autotune_form<double>(lp);
@@ -898,6 +928,8 @@ void scylla_lp::release() {
   h_done = nullptr;  // inside the h_ctl block
   if (arena) cudaFreeAsync(arena, st);  // to the pool, after the stream's work
   arena = nullptr;
+  if (arena_w) cudaFreeAsync(arena_w, st);
+  arena_w = nullptr;
   pinned_release(h_ctl);
   h_ctl = nullptr;
   if (ev_user) cudaEventDestroy(ev_user);
@@ -913,14 +945,20 @@ extern "C" int scylla_lp_create(const scylla_csr* A, const double* c, const doub
                                 const scylla_params* p, void* cuda_stream, scylla_lp** out) {
   if (!out) FAIL(SCYLLA_ERR_INVALID_ARG, "out is null");
   *out = nullptr;
-  int rc = validate_lp(A, c, row_lo, row_hi, col_lo, col_hi, is_integer);
+  // A small LP is validated here; a large one on the device once its arrays are there (on
+  // the bench workload the host's passes take 0.35 ms), and the host check runs only to
+  // report what is wrong, also when the device could not be used.
+  int rc = validate_structure(A, c, row_lo, row_hi, col_lo, col_hi, is_integer);
+  if (rc != SCYLLA_OK) return rc;
+  const bool big = A->nnz + 2 * (A->m + A->n) > 200000 && !(p && p->host_transpose);
+  if (!big) rc = validate_lp(A, c, row_lo, row_hi, col_lo, col_hi, is_integer);
   if (rc != SCYLLA_OK) return rc;
   scylla_params dp;
   scylla_default_params(&dp);
   scylla_lp* lp = nullptr;
   try {
     lp = new scylla_lp();
-    rc = create_impl(A, c, row_lo, row_hi, col_lo, col_hi, is_integer, p ? p : &dp, cuda_stream, lp);
+    rc = create_impl(A, c, row_lo, row_hi, col_lo, col_hi, is_integer, p ? p : &dp, cuda_stream, lp, big);
   } catch (const std::bad_alloc&) {
     set_error("host allocation failed");
     rc = SCYLLA_ERR_OOM;
@@ -929,10 +967,19 @@ extern "C" int scylla_lp_create(const scylla_csr* A, const double* c, const doub
     rc = SCYLLA_ERR_INVALID_ARG;
   }
   if (rc != SCYLLA_OK) {
+    const std::string why = get_error();
     if (lp) {
       lp->release();
       delete lp;
     }
+    if (big) {
+      try {
+        const int rv = validate_lp(A, c, row_lo, row_hi, col_lo, col_hi, is_integer);
+        if (rv != SCYLLA_OK) return rv;
+      } catch (const std::exception&) {
+      }
+    }
+    set_error(why);
     return rc;
   }
   *out = lp;
@@ -1601,7 +1648,7 @@ int scylla_lp::repair(const double* xhat, double tol, int64_t iter_limit, double
     q.precision = SCYLLA_PREC_FP64;
     q.infeasibility_checks = 0;  // the repair's screen proves infeasible fixings
     scylla_lp* r = new scylla_lp();
-    rc = create_impl(&A, c0.data(), lo0.data(), hi0.data(), l0.data(), u0.data(), int0.data(), &q, user_st, r);
+    rc = create_impl(&A, c0.data(), lo0.data(), hi0.data(), l0.data(), u0.data(), int0.data(), &q, user_st, r, false);
     if (rc != SCYLLA_OK) {
       r->release();
       delete r;

@@ -55,6 +55,7 @@ struct scylla_lp {
 
   void* arena = nullptr;
   size_t arena_bytes = 0;
+  void* arena_w = nullptr;  // wide tiles built after the arena (an L2-resident LP that is tuned after all)
   int *a_rowptr = nullptr, *a_cols = nullptr;
   int *t_rowptr = nullptr, *t_cols = nullptr;
   int2 *a_tiles = nullptr, *t_tiles = nullptr, *a_tiles_w = nullptr, *t_tiles_w = nullptr;

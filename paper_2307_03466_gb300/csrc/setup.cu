@@ -24,11 +24,8 @@ namespace {
 constexpr int kSetupThreads = 256;
 
 // lanes per row of a tile of nr rows: the largest power of two L with L * nr <= 32
-__device__ __forceinline__ int setup_row_lanes(int nr) {
-  if (nr >= 32) return 1;
-  const int l = 32 / (nr > 0 ? nr : 1);
-  return 1 << (31 - __clz(l));
-}
+// (its base-2 logarithm)
+__device__ __forceinline__ int setup_row_lanes_log2(int nr) { return nr >= 32 ? 0 : nr > 1 ? __clz(nr - 1) - 27 : 5; }
 
 int setup_grid(long long warps_or_items, int per_block) {
   long long g = (warps_or_items + per_block - 1) / per_block;
@@ -113,32 +110,75 @@ __global__ void k_column_kinds(long long n, const uint8_t* __restrict__ is_int, 
 //   (other_i |a_ij|) self_j on columns (the product order of the scaled values),
 // red = max for a Ruiz iteration and sum for the Pock-Chambolle step (alpha = 1);
 // a row without nonzeros keeps its factor.  The warp takes tiles t = first,
-// first + step, ...
+// first + step, ...; a tile's indices and values come into shared memory with consecutive
+// lanes on consecutive entries, and the lanes of a row then walk its entries there, eight
+// gathers ahead.  The maximum compares bit patterns (the terms are not negative), on the
+// integer pipe: an FP64 maximum costs several instructions of the slow FP64 pipe.
+constexpr int kSetupTile = kTileNnz;
+struct SetupStage {
+  double val[kSetupTile];
+  int idx[kSetupTile];
+};
 template <bool kMax, bool kRow>
 __device__ __forceinline__ void side_factor(int first, int step, const int2* __restrict__ tiles, int ntiles,
                                             const int* __restrict__ ptr, const int* __restrict__ idx,
                                             const double* __restrict__ vals, const double* __restrict__ self,
-                                            const double* __restrict__ other, double* __restrict__ out) {
+                                            const double* __restrict__ other, double* __restrict__ out,
+                                            SetupStage& S) {
+  constexpr int kAhead = 8;
   const int lane = threadIdx.x & 31;
   for (int t = first; t < ntiles; t += step) {
-    const int r0 = tiles[t].x, nr = tiles[t + 1].x - r0;
-    const int L = setup_row_lanes(nr), rl = lane / L, sub = lane - rl * L;
-    const bool mine = rl < nr;
-    const int row = r0 + rl;
-    double acc = 0.0, si = 0.0;
+    const int2 ta = tiles[t], tb = tiles[t + 1];
+    const int nr = tb.x - ta.x, p0 = ta.y, n = tb.y - ta.y;
+    const int sh = setup_row_lanes_log2(nr), L = 1 << sh, rl = lane >> sh, sub = lane & (L - 1);
+    const bool mine = rl < nr, staged = n <= kSetupTile;
+    const int row = ta.x + rl;
+    unsigned q0 = 0, q1 = 0;  // unsigned: a step past the longest row stays in range
+    double si = 0.0;
     if (mine) {
+      q0 = unsigned(ptr[row] - p0);
+      q1 = unsigned(ptr[row + 1] - p0);
       si = self[row];
-      const int q1 = ptr[row + 1];
-      for (int p = ptr[row] + sub; p < q1; p += L) {
-        const double a = fabs(vals[p]), o = other[idx[p]];
-        const double term = kRow ? (si * a) * o : (o * a) * si;
-        acc = kMax ? fmax(acc, term) : acc + term;
+    }
+    if (staged) {
+      __syncwarp();  // every lane is through with the last tile's entries
+#pragma unroll
+      for (int u = 0; u < kSetupTile / 32; ++u) {
+        const int q = lane + 32 * u;
+        if (q < n) {
+          S.idx[q] = idx[p0 + q];
+          S.val[q] = vals[p0 + q];
+        }
       }
+      __syncwarp();
+    }
+    constexpr long long kInfBits = 0x7ff0000000000000LL;
+    double acc = 0.0;
+    long long top = 0;  // the bits of the maximum
+    for (unsigned q = q0 + sub; q < q1; q += kAhead * L) {
+      double a[kAhead], o[kAhead];
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) {
+        const unsigned e = q + u * L;
+        if (e < q1) {
+          o[u] = other[staged ? S.idx[e] : idx[p0 + e]];
+          a[u] = fabs(staged ? S.val[e] : vals[p0 + e]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u)
+        if (q + u * L < q1) {
+          const double term = kRow ? (si * a[u]) * o[u] : (o[u] * a[u]) * si;
+          const long long bits = __double_as_longlong(term);
+          if (kMax) top = bits > top && bits <= kInfBits ? bits : top;  // a NaN is passed over, as by fmax
+          else acc += term;
+        }
     }
     for (int off = L >> 1; off > 0; off >>= 1) {
-      const double v = __shfl_down_sync(0xffffffffu, acc, off);
-      acc = kMax ? fmax(acc, v) : acc + v;
+      if (kMax) top = max(top, __shfl_down_sync(0xffffffffu, top, off));
+      else acc += __shfl_down_sync(0xffffffffu, acc, off);
     }
+    if (kMax) acc = __longlong_as_double(top);
     if (mine && sub == 0) out[row] = acc > 0.0 ? si / sqrt(acc) : si;
   }
 }
@@ -150,29 +190,28 @@ __global__ void __launch_bounds__(kSetupThreads) k_side_factors(DevSetup s, int 
                                                                const double* __restrict__ c, double* __restrict__ r2,
                                                                double* __restrict__ c2) {
   const int wpb = kSetupThreads / 32, w = int(threadIdx.x >> 5);
+  __shared__ SetupStage stage[kSetupThreads / 32];
   if (int(blockIdx.x) < gr) {
     side_factor<kMax, true>(int(blockIdx.x) * wpb + w, gr * wpb, s.a_tiles, s.a_ntiles, s.a_rowptr, s.a_cols,
-                            s.a_vals64, r, c, r2);
+                            s.a_vals64, r, c, r2, stage[w]);
   } else {
     const int b = int(blockIdx.x) - gr, gc = int(gridDim.x) - gr;
     side_factor<kMax, false>(b * wpb + w, gc * wpb, s.t_tiles, s.t_ntiles, s.t_rowptr, s.t_cols, s.t_vals64, c,
-                             r, c2);
+                             r, c2, stage[w]);
   }
 }
 
 // a~_ij = (a_ij R_i) C_j in place on one side (kRow: A, self = R; else A^T, self =
 // C), with the FP32 shadow when vals32 is given; both sides round the same product.
 template <bool kRow>
-__global__ void __launch_bounds__(kSetupThreads)
-    k_scale_side(const int2* __restrict__ tiles, int ntiles, const int* __restrict__ ptr, const int* __restrict__ idx,
-                 double* __restrict__ vals, float* __restrict__ vals32, const double* __restrict__ self,
-                 const double* __restrict__ other) {
+__device__ __forceinline__ void scale_side(int first, int step, const int2* __restrict__ tiles, int ntiles,
+                                           const int* __restrict__ ptr, const int* __restrict__ idx,
+                                           double* __restrict__ vals, float* __restrict__ vals32,
+                                           const double* __restrict__ self, const double* __restrict__ other) {
   const int lane = threadIdx.x & 31;
-  const int warp = int((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nwarps = int((gridDim.x * blockDim.x) >> 5);
-  for (int t = warp; t < ntiles; t += nwarps) {
+  for (int t = first; t < ntiles; t += step) {
     const int r0 = tiles[t].x, nr = tiles[t + 1].x - r0;
-    const int L = setup_row_lanes(nr), rl = lane / L, sub = lane - rl * L;
+    const int sh = setup_row_lanes_log2(nr), L = 1 << sh, rl = lane >> sh, sub = lane & (L - 1);
     if (rl >= nr) continue;
     const int row = r0 + rl;
     const double si = self[row];
@@ -183,6 +222,17 @@ __global__ void __launch_bounds__(kSetupThreads)
       vals[p] = v;
       if (vals32) vals32[p] = float(v);
     }
+  }
+}
+__global__ void __launch_bounds__(kSetupThreads) k_scale_sides(DevSetup s, int gr) {
+  const int wpb = kSetupThreads / 32, w = int(threadIdx.x >> 5);
+  if (int(blockIdx.x) < gr) {
+    scale_side<true>(int(blockIdx.x) * wpb + w, gr * wpb, s.a_tiles, s.a_ntiles, s.a_rowptr, s.a_cols, s.a_vals64,
+                     s.a_vals32, s.R, s.C);
+  } else {
+    const int b = int(blockIdx.x) - gr, gc = int(gridDim.x) - gr;
+    scale_side<false>(b * wpb + w, gc * wpb, s.t_tiles, s.t_ntiles, s.t_rowptr, s.t_cols, s.t_vals64, s.t_vals32, s.C,
+                      s.R);
   }
 }
 
@@ -226,7 +276,52 @@ void side_factors(const DevSetup& s, double* r, double* c, double* r2, double* c
   k_side_factors<kMax><<<gr + gc, kSetupThreads, 0, st>>>(s, gr, r, c, r2, c2);
 }
 
+// Whether an LP's arrays are malformed, as scylla_lp_create's host check finds it (which
+// names the place): column indices out of range or not increasing within a row, values or
+// costs not finite, bounds NaN, crossed or infinite on the wrong side, an integrality flag
+// other than 0 and 1, an integer column with a fractional finite bound.  rowptr is already
+// known to be non-decreasing from 0 to nnz.
+__global__ void k_malformed(int m, int n, int nnz, const int* __restrict__ rowptr, const int* __restrict__ cols,
+                            const double* __restrict__ vals, const double* __restrict__ c,
+                            const double* __restrict__ lo, const double* __restrict__ hi, const double* __restrict__ l,
+                            const double* __restrict__ u, const uint8_t* __restrict__ is_int, int* __restrict__ bad) {
+  const double inf = __longlong_as_double(0x7ff0000000000000LL);
+  const long long stride = (long long)gridDim.x * blockDim.x, t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  bool w = false;
+  for (long long p = t0; p < nnz; p += stride) {
+    const int j = cols[p];
+    w = w || j < 0 || j >= n || !isfinite(vals[p]);
+    if (p > 0 && cols[p - 1] >= j) {  // a row must start here: some rowptr entry is p
+      int a = 0, b = m;
+      while (a < b) {
+        const int mid = a + ((b - a) >> 1);
+        if (rowptr[mid] < p) a = mid + 1;
+        else b = mid;
+      }
+      w = w || rowptr[a] != p;
+    }
+  }
+  auto bounds = [&](double a, double b) { return isnan(a) || isnan(b) || a > b || a == inf || b == -inf; };
+  for (long long i = t0; i < m; i += stride) w = w || bounds(lo[i], hi[i]);
+  for (long long j = t0; j < n; j += stride) {
+    const uint8_t k = is_int[j];
+    w = w || !isfinite(c[j]) || bounds(l[j], u[j]) || k > 1 ||
+        (k && ((isfinite(l[j]) && l[j] != floor(l[j])) || (isfinite(u[j]) && u[j] != floor(u[j]))));
+  }
+  if (w) *bad = 1;
+}
+
 }  // namespace
+
+cudaError_t check_malformed(int m, int n, int nnz, const int* rowptr, const int* cols, const double* vals,
+                            const double* c, const double* lo, const double* hi, const double* l, const double* u,
+                            const uint8_t* is_int, int* bad, cudaStream_t st) {
+  long long work = nnz > n ? nnz : n;
+  if (m > work) work = m;
+  k_malformed<<<setup_grid(work, kSetupThreads), kSetupThreads, 0, st>>>(m, n, nnz, rowptr, cols, vals, c, lo, hi, l, u,
+                                                                         is_int, bad);
+  return cudaGetLastError();
+}
 
 cudaError_t fill_f64(double* p, long long count, double v, cudaStream_t st) {
   if (count > 0) k_fill_f64<<<setup_grid(count, kSetupThreads), kSetupThreads, 0, st>>>(p, count, v);
@@ -298,10 +393,7 @@ cudaError_t launch_precondition(const DevSetup& s, int ruiz_iters, bool pock_cha
 
 cudaError_t launch_scale_values(const DevSetup& s, cudaStream_t st) {
   const int gr = setup_grid(s.a_ntiles, kSetupThreads / 32), gc = setup_grid(s.t_ntiles, kSetupThreads / 32);
-  k_scale_side<true><<<gr, kSetupThreads, 0, st>>>(s.a_tiles, s.a_ntiles, s.a_rowptr, s.a_cols, s.a_vals64,
-                                                   s.a_vals32, s.R, s.C);
-  k_scale_side<false><<<gc, kSetupThreads, 0, st>>>(s.t_tiles, s.t_ntiles, s.t_rowptr, s.t_cols, s.t_vals64,
-                                                    s.t_vals32, s.C, s.R);
+  k_scale_sides<<<gr + gc, kSetupThreads, 0, st>>>(s, gr);
   return cudaGetLastError();
 }
 
