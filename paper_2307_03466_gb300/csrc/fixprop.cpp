@@ -99,6 +99,11 @@ struct Propagator {
     }
   }
 
+  // the row records that fixing column j will touch
+  void prefetch(int64_t j) const {
+    for (int64_t q = lp.colptr0[j]; q < lp.colptr0[j + 1]; ++q) __builtin_prefetch(&rows[size_t(lp.colrows0[q])], 1);
+  }
+
   int32_t pop() {
     const int32_t i = ring[size_t(head)];
     if (++head == lp.m0) head = 0;
@@ -363,25 +368,50 @@ bool check_feasible_host(const scylla_lp& lp, const double* x) {
 
 namespace {
 
+// The integer columns by (distance of xbar to its rounding, index).  At an LP point most
+// distances are exactly 0: those columns come first, in index order, and only the others
+// are sorted, as (distance, index) pairs (packing/covering 8000 x 20,000 with 8000 binaries:
+// the comparisons through an index array had been a third of the call).
+std::vector<int32_t> fixing_order(const scylla_lp& lp, const double* xbar) {
+  std::vector<int32_t> order;
+  order.reserve(size_t(lp.n_int));
+  std::vector<std::pair<double, int32_t>> rest;
+  bool finite = true;
+  for (int64_t j = 0; j < lp.n0; ++j) {
+    if (!lp.int0[j]) continue;
+    const double d = std::fabs(xbar[j] - round_half_up(xbar[j]));
+    finite = finite && std::isfinite(d);
+    if (d == 0.0) order.push_back(int32_t(j));
+    else rest.emplace_back(d, int32_t(j));
+  }
+  auto before = [](const std::pair<double, int32_t>& a, const std::pair<double, int32_t>& b) {
+    return a.first != b.first ? a.first < b.first : a.second < b.second;
+  };
+  if (finite) {
+    std::sort(rest.begin(), rest.end(), before);
+  } else {
+    // an infinite entry has no distance: the order of the comparison sort over every column
+    std::vector<std::pair<double, int32_t>> all;
+    for (int64_t j = 0; j < lp.n0; ++j)
+      if (lp.int0[j]) all.emplace_back(std::fabs(xbar[j] - round_half_up(xbar[j])), int32_t(j));
+    std::stable_sort(all.begin(), all.end(), before);
+    order.clear();
+    rest.swap(all);
+  }
+  for (const auto& p : rest) order.push_back(p.second);
+  return order;
+}
+
 // the fixing loop for one point, from the kept first propagation (read only, so that
 // several points can run at once)
 void fix_one(const scylla_lp& lp, const RootState& root, const double* xbar, double* xhat, double* dom_lo,
              double* dom_hi, int32_t* fixed_cols, int64_t* n_fixed, uint8_t* ignored_rows) {
   Propagator pr(lp, root.dom, root.rows);
-  std::vector<int64_t> order;
-  order.reserve(size_t(lp.n_int));
-  std::vector<double> dist(size_t(lp.n0), 0.0);
-  for (int64_t j = 0; j < lp.n0; ++j) {
-    if (!lp.int0[j]) continue;
-    order.push_back(j);
-    dist[j] = std::fabs(xbar[j] - round_half_up(xbar[j]));
-  }
-  std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) {
-    if (dist[a] != dist[b]) return dist[a] < dist[b];
-    return a < b;
-  });
+  const std::vector<int32_t> order = fixing_order(lp, xbar);
   int64_t nf = 0;
-  for (int64_t j : order) {
+  for (size_t k = 0; k < order.size(); ++k) {
+    const int64_t j = order[k];
+    if (k + 2 < order.size()) pr.prefetch(order[k + 2]);
     Propagator::Dom& d = pr.dom[size_t(j)];
     if (d.lb == d.ub) continue;
     double v = round_half_up(xbar[j]);
