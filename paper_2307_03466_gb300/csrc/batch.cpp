@@ -35,6 +35,7 @@ struct scylla_batch {
   cudaEvent_t ev_user = nullptr, ev0 = nullptr, ev1 = nullptr;
   cudaEvent_t ev_chunk[2] = {nullptr, nullptr};
   int* h_done = nullptr;  // pinned, two slots
+  double* h_io = nullptr;  // pinned, kReadStage doubles behind h_done (read_back)
   int nlp = 0;
   std::vector<int> row_off, col_off;  // per LP (nlp + 1)
   int m = 0, n = 0, nnz = 0;
@@ -68,6 +69,7 @@ struct scylla_batch {
     h_ctl = nullptr;
     if (h_done) cudaFreeHost(h_done);
     h_done = nullptr;
+    h_io = nullptr;
     if (h_err) cudaFreeHost(h_err);
     h_err = nullptr;
     for (cudaEvent_t* e : {&ev_user, &ev0, &ev1, &ev_chunk[0], &ev_chunk[1]}) {
@@ -260,7 +262,8 @@ int create_batch(int32_t count, const scylla_csr* A, const double* const* c, con
   CKB(cudaStreamCreateWithFlags(&h->st, cudaStreamNonBlocking));
   for (cudaEvent_t* e : {&h->ev_user, &h->ev0, &h->ev1}) CKB(cudaEventCreate(e));
   for (int k = 0; k < 2; ++k) CKB(cudaEventCreateWithFlags(&h->ev_chunk[k], cudaEventDisableTiming));
-  CKB(cudaMallocHost(&h->h_done, 2 * sizeof(int)));
+  CKB(cudaMallocHost(&h->h_done, 64 + sizeof(double) * kReadStage));
+  h->h_io = reinterpret_cast<double*>(reinterpret_cast<char*>(h->h_done) + 64);
   CKB(cudaMallocHost(&h->h_err, sizeof(int)));
 
   // ---- block-diagonal LP
@@ -775,10 +778,10 @@ extern "C" int scylla_batch_get_primal(const scylla_batch* h, int32_t b, double*
   }
   const int c0 = h->col_off[b], cnt = h->col_off[b + 1] - h->col_off[b];
   cudaStream_t st = h->st;
-  if (h->p.precision == SCYLLA_PREC_MIXED) CKB(launch_batch_get_x<float>(h->b32, b, c0, cnt, h->io, st));
-  else CKB(launch_batch_get_x<double>(h->b64, b, c0, cnt, h->io, st));
-  CKB(cudaMemcpyAsync(x, h->io, sizeof(double) * cnt, cudaMemcpyDeviceToHost, st));
-  CKB(cudaStreamSynchronize(st));
+  CKB(read_back(x, cnt, h->io, h->h_io, st, [&](double* out) {
+    return h->p.precision == SCYLLA_PREC_MIXED ? launch_batch_get_x<float>(h->b32, b, c0, cnt, out, st)
+                                               : launch_batch_get_x<double>(h->b64, b, c0, cnt, out, st);
+  }));
   return SCYLLA_OK;
 }
 
@@ -792,10 +795,10 @@ extern "C" int scylla_batch_get_dual(const scylla_batch* h, int32_t b, double* y
   const int r0 = h->row_off[b], cnt = h->row_off[b + 1] - h->row_off[b];
   if (cnt == 0) return SCYLLA_OK;
   cudaStream_t st = h->st;
-  if (h->p.precision == SCYLLA_PREC_MIXED) CKB(launch_batch_get_y<float>(h->b32, b, r0, cnt, h->io, st));
-  else CKB(launch_batch_get_y<double>(h->b64, b, r0, cnt, h->io, st));
-  CKB(cudaMemcpyAsync(y, h->io, sizeof(double) * size_t(cnt), cudaMemcpyDeviceToHost, st));
-  CKB(cudaStreamSynchronize(st));
+  CKB(read_back(y, cnt, h->io, h->h_io, st, [&](double* out) {
+    return h->p.precision == SCYLLA_PREC_MIXED ? launch_batch_get_y<float>(h->b32, b, r0, cnt, out, st)
+                                               : launch_batch_get_y<double>(h->b64, b, r0, cnt, out, st);
+  }));
   return SCYLLA_OK;
 }
 

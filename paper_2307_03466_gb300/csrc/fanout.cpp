@@ -33,6 +33,7 @@ struct scylla_fanout {
   std::vector<Control> ctl0;
   Control* h_ctl = nullptr;
   int* h_done = nullptr;
+  double* h_io = nullptr;  // pinned, kReadStage doubles behind h_done (read_back)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_chunk[2] = {nullptr, nullptr};
   DevFan<double> f64{};
   DevFan<float> f32{};
@@ -57,6 +58,7 @@ struct scylla_fanout {
     h_ctl = nullptr;
     if (h_done) cudaFreeHost(h_done);
     h_done = nullptr;
+    h_io = nullptr;
     for (cudaEvent_t* e : {&ev0, &ev1, &ev_chunk[0], &ev_chunk[1]}) {
       if (*e) cudaEventDestroy(*e);
       *e = nullptr;
@@ -192,7 +194,8 @@ int create_fan(scylla_lp* lp, int K, const double* targets, int round_K, scylla_
   const int64_t n0 = lp->n0;
   for (cudaEvent_t* e : {&f->ev0, &f->ev1}) CKF(cudaEventCreate(e));
   for (int q = 0; q < 2; ++q) CKF(cudaEventCreateWithFlags(&f->ev_chunk[q], cudaEventDisableTiming));
-  CKF(cudaMallocHost(&f->h_done, 2 * sizeof(int)));
+  CKF(cudaMallocHost(&f->h_done, 64 + sizeof(double) * kReadStage));
+  f->h_io = reinterpret_cast<double*>(reinterpret_cast<char*>(f->h_done) + 64);
   CKF(cudaMallocHost(&f->h_ctl, sizeof(Control) * K));
   // the objective of target k (Section 2.4, round round_K): c_hat = t c + om g_k
   const double aK = std::pow(lp->p.alpha, double(round_K));
@@ -544,10 +547,10 @@ extern "C" int scylla_fanout_get_primal(const scylla_fanout* f, int32_t k, doubl
     return SCYLLA_ERR_INVALID_ARG;
   }
   cudaStream_t st = f->lp->st;
-  if (f->lp->p.precision == SCYLLA_PREC_MIXED) CKF(launch_fan_get_x<float>(f->f32, k, f->io, st));
-  else CKF(launch_fan_get_x<double>(f->f64, k, f->io, st));
-  CKF(cudaMemcpyAsync(x, f->io, sizeof(double) * f->lp->n0, cudaMemcpyDeviceToHost, st));
-  CKF(cudaStreamSynchronize(st));
+  CKF(read_back(x, int(f->lp->n0), f->io, f->h_io, st, [&](double* out) {
+    return f->lp->p.precision == SCYLLA_PREC_MIXED ? launch_fan_get_x<float>(f->f32, k, out, st)
+                                                   : launch_fan_get_x<double>(f->f64, k, out, st);
+  }));
   return SCYLLA_OK;
 }
 
@@ -557,10 +560,10 @@ extern "C" int scylla_fanout_get_dual(const scylla_fanout* f, int32_t k, double*
     return SCYLLA_ERR_INVALID_ARG;
   }
   cudaStream_t st = f->lp->st;
-  if (f->lp->p.precision == SCYLLA_PREC_MIXED) CKF(launch_fan_get_y<float>(f->f32, k, f->io, st));
-  else CKF(launch_fan_get_y<double>(f->f64, k, f->io, st));
-  CKF(cudaMemcpyAsync(y, f->io, sizeof(double) * f->lp->m0, cudaMemcpyDeviceToHost, st));
-  CKF(cudaStreamSynchronize(st));
+  CKF(read_back(y, int(f->lp->m0), f->io, f->h_io, st, [&](double* out) {
+    return f->lp->p.precision == SCYLLA_PREC_MIXED ? launch_fan_get_y<float>(f->f32, k, out, st)
+                                                   : launch_fan_get_y<double>(f->f64, k, out, st);
+  }));
   return SCYLLA_OK;
 }
 

@@ -1642,9 +1642,15 @@ __global__ void k_set_xy(DevLP<T> d, const double* x, const double* y) {
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < d.n; j += stride) xc[j] = T(x[j] / d.C[j]);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.m; i += stride) yc[i] = T(y[i] / d.R[i]);
 }
-// x = proj_[l,u](0), y = 0 (Algorithm 1 initialisation, x projected onto its box)
+// x = proj_[l,u](0), y = 0 (Algorithm 1 initialisation, x projected onto its box), and
+// with `set` the step size and primal weight (a copy of the control block to the host and
+// back took a wait more)
 template <typename T>
-__global__ void k_init_point(DevLP<T> d) {
+__global__ void k_init_point(DevLP<T> d, bool set, double eta, double omega) {
+  if (set && blockIdx.x == 0 && threadIdx.x == 0) {
+    d.ctl->eta = eta;
+    d.ctl->omega = omega;
+  }
   T* xc = d.X[d.ctl->ix_cur];
   T* yc = d.Y[d.ctl->ix_cur];
   const int stride = gridDim.x * blockDim.x;
@@ -2969,8 +2975,10 @@ static cudaError_t launch_step_kernel(void (*kernel)(DevLP<T>), int grid, const 
 }
 
 template <typename T>
-cudaError_t launch_check(const DevLP<T>& d, cudaStream_t st) {
-  cudaError_t e = launch_step_kernel<T>(d.q64 ? k_check_cols<T, 1> : k_check_cols<T, 0>, d.grid_c1, d, st);
+cudaError_t launch_check(const DevLP<T>& d, cudaStream_t st, bool after_step) {
+  DevLP<T> dc = d;
+  if (!after_step) dc.pdl = 0;
+  cudaError_t e = launch_step_kernel<T>(d.q64 ? k_check_cols<T, 1> : k_check_cols<T, 0>, d.grid_c1, dc, st);
   // infeasibility detection: the ray's terms, before the row half takes the decision
   if (e == cudaSuccess && d.inf_cand) e = launch_infeas<T>(d, st);
   if (e == cudaSuccess) e = launch_step_kernel<T>(k_check_rows<T>, d.grid_c2, d, st);
@@ -3038,8 +3046,10 @@ cudaError_t launch_set_xy(const DevLP<T>& d, const double* x, const double* y, c
   return cudaGetLastError();
 }
 template <typename T>
-cudaError_t launch_init_point(const DevLP<T>& d, cudaStream_t st) {
-  k_init_point<T><<<ew_grid(d.m > d.n ? d.m : d.n), kThreads, 0, st>>>(d);
+cudaError_t launch_init_point(const DevLP<T>& d, cudaStream_t st, const double* eta_omega) {
+  k_init_point<T><<<ew_grid(d.m > d.n ? d.m : d.n), kThreads, 0, st>>>(d, eta_omega != nullptr,
+                                                                       eta_omega ? eta_omega[0] : 0.0,
+                                                                       eta_omega ? eta_omega[1] : 0.0);
   return cudaGetLastError();
 }
 
@@ -3107,7 +3117,7 @@ int occupancy_grid(int side, int form, int work_tiles) {
 
 #define SCYLLA_INSTANTIATE(T)                                                                              \
   template cudaError_t launch_solve_init<T>(const DevLP<T>&, double, long long, int, long long, cudaStream_t); \
-  template cudaError_t launch_check<T>(const DevLP<T>&, cudaStream_t);                                    \
+  template cudaError_t launch_check<T>(const DevLP<T>&, cudaStream_t, bool);                              \
   template cudaError_t launch_slot<T>(const DevLP<T>&, cudaStream_t);                                     \
   template cudaError_t launch_primal<T>(const DevLP<T>&, cudaStream_t);                                   \
   template cudaError_t launch_dual<T>(const DevLP<T>&, cudaStream_t);                                     \
@@ -3116,7 +3126,7 @@ int occupancy_grid(int side, int form, int work_tiles) {
   template cudaError_t launch_get_x<T>(const DevLP<T>&, double*, int, cudaStream_t);                      \
   template cudaError_t launch_get_y<T>(const DevLP<T>&, double*, int, cudaStream_t);                      \
   template cudaError_t launch_set_xy<T>(const DevLP<T>&, const double*, const double*, cudaStream_t);     \
-  template cudaError_t launch_init_point<T>(const DevLP<T>&, cudaStream_t);                               \
+  template cudaError_t launch_init_point<T>(const DevLP<T>&, cudaStream_t, const double*);                \
   template int occupancy_grid<T>(int, int, int);                                                           \
   template int persistent_blocks_per_sm<T>();                                                             \
   template bool resident_plan<T>(const DevLP<T>&, ResidentPlan*);                                         \

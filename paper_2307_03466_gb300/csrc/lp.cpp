@@ -133,9 +133,12 @@ cudaError_t handle_pool(int device, cudaMemPool_t* out) {
   return cudaSuccess;
 }
 
-// Pinned host blocks of kPinnedBlock bytes (a handle's control-block mirror and
-// done flags), kept on a free list for reuse instead of cudaFreeHost.
-constexpr size_t kPinnedBlock = sizeof(scylla::Control) + 64;
+// Pinned host blocks of a handle, kept on a free list for reuse instead of cudaFreeHost.
+struct PinnedBlock {
+  scylla::Control ctl, chunk[2];
+  int flag;
+  alignas(64) double x[scylla::kReadStage], y[scylla::kReadStage];
+};
 std::mutex g_pinned_mu;
 std::vector<void*> g_pinned_free;
 
@@ -148,7 +151,7 @@ cudaError_t pinned_acquire(void** p) {
       return cudaSuccess;
     }
   }
-  return cudaMallocHost(p, kPinnedBlock);
+  return cudaMallocHost(p, sizeof(PinnedBlock));
 }
 
 void pinned_release(void* p) {
@@ -645,14 +648,17 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
   cudaStream_t st = lp->st;
   CK(cudaMemsetAsync(lp->arena, 0, lp->arena_bytes, st));
   {
-    // one pinned block: the control block's host copy, then the two done flags
     void* pin = nullptr;
     CK(pinned_acquire(&pin));
-    lp->h_ctl = static_cast<Control*>(pin);
-    lp->h_done = reinterpret_cast<int*>(static_cast<char*>(pin) + sizeof(Control));
+    PinnedBlock* b = static_cast<PinnedBlock*>(pin);
+    lp->h_ctl = &b->ctl;  // the block's start: released by this address
+    lp->h_chunk = b->chunk;
+    lp->h_flag = &b->flag;
+    lp->h_x = b->x;
+    lp->h_y = b->y;
   }
-  CK(cudaEventCreateWithFlags(&lp->ev_chunk[0], cudaEventDisableTiming));
-  CK(cudaEventCreateWithFlags(&lp->ev_chunk[1], cudaEventDisableTiming));
+  CK(cudaEventCreate(&lp->ev_chunk[0]));
+  CK(cudaEventCreate(&lp->ev_chunk[1]));
 
   CK(cudaMemcpyAsync(lp->a_rowptr, rp.data(), sizeof(int) * (m + 1), cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(lp->a_cols, ci, sizeof(int) * nnz, cudaMemcpyHostToDevice, st));
@@ -672,9 +678,9 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
     int* bad = reinterpret_cast<int*>(lp->red_c1);  // zero from the arena's clearing
     CK(check_malformed(int(m0), int(n0), int(nnz0), lp->a_rowptr, lp->a_cols, lp->a_vals64, lp->c_un, lp->lo_un,
                        lp->hi_un, lp->l_un, lp->u_un, lp->int_mask, bad, st));
-    CK(cudaMemcpyAsync(lp->h_done, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(lp->h_flag, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    if (lp->h_done[0] != 0) FAIL(SCYLLA_ERR_INVALID_ARG, "malformed LP");  // the host check says where
+    if (*lp->h_flag != 0) FAIL(SCYLLA_ERR_INVALID_ARG, "malformed LP");  // the host check says where
   }
   if (host_tp) {
     CK(cudaMemcpyAsync(lp->t_rowptr, tp.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, st));
@@ -925,7 +931,9 @@ void scylla_lp::release() {
     if (e) cudaEventDestroy(e);
     e = nullptr;
   }
-  h_done = nullptr;  // inside the h_ctl block
+  h_chunk = nullptr;  // inside the h_ctl block
+  h_flag = nullptr;
+  h_x = h_y = nullptr;
   if (arena) cudaFreeAsync(arena, st);  // to the pool, after the stream's work
   arena = nullptr;
   if (arena_w) cudaFreeAsync(arena_w, st);
@@ -935,7 +943,7 @@ void scylla_lp::release() {
   if (ev_user) cudaEventDestroy(ev_user);
   if (ev0) cudaEventDestroy(ev0);
   if (ev1) cudaEventDestroy(ev1);
-  ev_user = ev0 = ev1 = nullptr;
+  ev_user = ev0 = ev1 = ev_end = nullptr;
   if (st) cudaStreamDestroy(st);
   st = nullptr;
 }
@@ -1061,9 +1069,7 @@ static int build_chunk_graph(scylla_lp* lp, const DevLP<T>& d) {
   cudaError_t e = cudaSuccess;
   if (lp->resident.scope) {
     e = launch_attempts<T>(d, lp->resident, lp->grid_bar, st);
-    DevLP<T> dc = d;
-    dc.pdl = 0;  // its predecessor is not a launch that triggers its successor
-    if (e == cudaSuccess) e = launch_check<T>(dc, st);
+    if (e == cudaSuccess) e = launch_check<T>(d, st, false);
   } else {
     for (int s = 0; s < lp->p.n_check && e == cudaSuccess; ++s) e = launch_slot<T>(d, st);
     if (e == cudaSuccess) e = launch_check<T>(d, st);
@@ -1091,6 +1097,7 @@ static int solve_impl(scylla_lp* lp, const DevLP<T>& d, double tol, int64_t iter
   cudaStream_t st = lp->st;
   const long long nchk = lp->p.n_check;
   const long long max_chunks = (iter_limit + nchk - 1) / nchk + 2;
+  lp->ev_end = lp->ev1;
   CK(cudaEventRecord(lp->ev0, st));
   CK(launch_solve_init<T>(d, tol, (long long)iter_limit, stall_checks, max_chunks, st));
   long long launches = 1;
@@ -1122,11 +1129,13 @@ static int solve_impl(scylla_lp* lp, const DevLP<T>& d, double tol, int64_t iter
       if (rc != SCYLLA_OK) return rc;
     }
     // chunk c+1 is queued before the done flag of chunk c is read, so the GPU never
-    // waits for the host; the chunk queued after the last one returns at once
+    // waits for the host; the chunk queued after the last one returns at once.  A chunk's
+    // whole control block comes back, so that a solve whose last chunk has no successor
+    // ends with that copy and its event.
     auto enqueue = [&](long long c) -> cudaError_t {
       cudaError_t e = cudaGraphLaunch(lp->chunk_exec, st);
       if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&lp->h_done[c & 1], &lp->ctl->done, sizeof(int), cudaMemcpyDeviceToHost, st);
+        e = cudaMemcpyAsync(&lp->h_chunk[c & 1], lp->ctl, sizeof(Control), cudaMemcpyDeviceToHost, st);
       if (e == cudaSuccess) e = cudaEventRecord(lp->ev_chunk[c & 1], st);
       launches += per_chunk;
       return e;
@@ -1138,7 +1147,13 @@ static int solve_impl(scylla_lp* lp, const DevLP<T>& d, double tol, int64_t iter
       const bool ahead = c + 1 < need;
       if (ahead) CK(enqueue(c + 1));
       CK(cudaEventSynchronize(lp->ev_chunk[c & 1]));
-      if (lp->h_done[c & 1]) break;
+      if (lp->h_chunk[c & 1].done) {
+        if (ahead) break;
+        *lp->h_ctl = lp->h_chunk[c & 1];
+        lp->ev_end = lp->ev_chunk[c & 1];
+        lp->last_launches = launches;
+        return SCYLLA_OK;
+      }
       if (!ahead && c + 1 < max_chunks) CK(enqueue(c + 1));
     }
   } else {
@@ -1201,7 +1216,7 @@ int scylla_lp::solve(double tol, int64_t iter_limit, int stall_checks, scylla_pd
     out->eta = h.eta;
     out->omega = h.omega;
     float ms = 0.f;
-    cudaEventElapsedTime(&ms, ev0, ev1);
+    cudaEventElapsedTime(&ms, ev0, ev_end);
     out->seconds = ms * 1e-3;
     out->launches = last_launches >= 0 ? last_launches : 3 + h.chunks * (2LL * p.n_check + 3);
     out->kernel_form = api_form(form_p);
@@ -1278,21 +1293,31 @@ extern "C" int scylla_get_objective(const scylla_lp* lp, double* c_hat, double* 
 
 // ------------------------------------------------------------- state access ---
 int scylla_lp::fetch_x(double* host, int count) {
-  if (p.precision == SCYLLA_PREC_MIXED) CK(launch_get_x<float>(d32, io_x, count, st));
-  else CK(launch_get_x<double>(d64, io_x, count, st));
-  if (host) {
-    CK(cudaMemcpyAsync(host, io_x, sizeof(double) * count, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-  }
+  auto get = [&](double* out) {
+    return p.precision == SCYLLA_PREC_MIXED ? launch_get_x<float>(d32, out, count, st)
+                                            : launch_get_x<double>(d64, out, count, st);
+  };
+  if (host) CK(read_back(host, count, io_x, h_x, st, get));
+  else CK(get(io_x));
   return SCYLLA_OK;
 }
 
 int scylla_lp::fetch_y(double* host, int count) {
-  if (p.precision == SCYLLA_PREC_MIXED) CK(launch_get_y<float>(d32, io_y, count, st));
-  else CK(launch_get_y<double>(d64, io_y, count, st));
-  CK(cudaMemcpyAsync(host, io_y, sizeof(double) * count, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
+  auto get = [&](double* out) {
+    return p.precision == SCYLLA_PREC_MIXED ? launch_get_y<float>(d32, out, count, st)
+                                            : launch_get_y<double>(d64, out, count, st);
+  };
+  CK(read_back(host, count, io_y, h_y, st, get));
   return SCYLLA_OK;
+}
+
+bool scylla::pageable_host(const void* host) {
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeUnregistered || a.type == cudaMemoryTypeHost;
 }
 
 extern "C" int scylla_get_certificate(const scylla_lp* lp, double* y, double* gap, double* scale) {
@@ -1728,13 +1753,9 @@ extern "C" int scylla_reset_state(scylla_lp* lp) {
   int rc = lp->order_after_user();
   if (rc != SCYLLA_OK) return rc;
   cudaStream_t st = lp->st;
-  if (lp->p.precision == SCYLLA_PREC_MIXED) CK(launch_init_point<float>(lp->d32, st));
-  else CK(launch_init_point<double>(lp->d64, st));
-  CK(cudaMemcpyAsync(lp->h_ctl, lp->ctl, sizeof(Control), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  lp->h_ctl->eta = lp->eta0;
-  lp->h_ctl->omega = lp->omega0;
-  CK(cudaMemcpyAsync(lp->ctl, lp->h_ctl, sizeof(Control), cudaMemcpyHostToDevice, st));
+  const double eta_omega[2] = {lp->eta0, lp->omega0};
+  if (lp->p.precision == SCYLLA_PREC_MIXED) CK(launch_init_point<float>(lp->d32, st, eta_omega));
+  else CK(launch_init_point<double>(lp->d64, st, eta_omega));
   CK(cudaStreamSynchronize(st));
   return SCYLLA_OK;
 }

@@ -15,6 +15,7 @@ struct scylla_lp {
   cudaStream_t st = nullptr;       // the handle's own stream (graphs are captured on it)
   cudaStream_t user_st = nullptr;  // caller's stream: its prior work is ordered before each call
   cudaEvent_t ev_user = nullptr, ev0 = nullptr, ev1 = nullptr;
+  cudaEvent_t ev_end = nullptr;  // the event that ended the last solve: ev1 or one of ev_chunk
 
   // original MIP on the host (fix-and-propagate, feasibility test, run loop)
   int64_t m0 = 0, n0 = 0, nnz0 = 0;
@@ -113,7 +114,9 @@ struct scylla_lp {
   cudaGraph_t chunk_graph = nullptr;  // n_check attempts + one check (use_graph = 1)
   cudaGraphExec_t chunk_exec = nullptr;
   cudaEvent_t ev_chunk[2] = {nullptr, nullptr};
-  int* h_done = nullptr;             // pinned, two slots
+  scylla::Control* h_chunk = nullptr;  // pinned: the control block after a chunk, two slots
+  int* h_flag = nullptr;               // pinned
+  double *h_x = nullptr, *h_y = nullptr;  // pinned, kReadStage doubles each (read_back)
   int64_t last_launches = 0;
 
   // the continuous-repair copy of the original MIP (scylla_repair), built on first use
