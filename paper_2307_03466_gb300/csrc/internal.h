@@ -323,7 +323,7 @@ cudaError_t read_back(double* host, int count, double* dev, double* stage, cudaS
   return e;
 }
 cudaError_t fill_f64(double* p, long long count, double v, cudaStream_t st);
-// *bad = 1 when the arrays are malformed (scylla_lp_create); bad is cleared by the caller
+// the arrays are malformed unless bad[0] and bad[1] stay 0 (scylla_lp_create); cleared by the caller
 cudaError_t check_malformed(int m, int n, int nnz, const int* rowptr, const int* cols, const double* vals,
                             const double* c, const double* lo, const double* hi, const double* l, const double* u,
                             const uint8_t* is_int, int* bad, cudaStream_t st);

@@ -136,7 +136,7 @@ cudaError_t handle_pool(int device, cudaMemPool_t* out) {
 // Pinned host blocks of a handle, kept on a free list for reuse instead of cudaFreeHost.
 struct PinnedBlock {
   scylla::Control ctl, chunk[2];
-  int flag;
+  int flag[2];
   alignas(64) double x[scylla::kReadStage], y[scylla::kReadStage];
 };
 std::mutex g_pinned_mu;
@@ -653,7 +653,7 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
     PinnedBlock* b = static_cast<PinnedBlock*>(pin);
     lp->h_ctl = &b->ctl;  // the block's start: released by this address
     lp->h_chunk = b->chunk;
-    lp->h_flag = &b->flag;
+    lp->h_flag = b->flag;
     lp->h_x = b->x;
     lp->h_y = b->y;
   }
@@ -678,9 +678,9 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
     int* bad = reinterpret_cast<int*>(lp->red_c1);  // zero from the arena's clearing
     CK(check_malformed(int(m0), int(n0), int(nnz0), lp->a_rowptr, lp->a_cols, lp->a_vals64, lp->c_un, lp->lo_un,
                        lp->hi_un, lp->l_un, lp->u_un, lp->int_mask, bad, st));
-    CK(cudaMemcpyAsync(lp->h_flag, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(lp->h_flag, bad, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    if (*lp->h_flag != 0) FAIL(SCYLLA_ERR_INVALID_ARG, "malformed LP");  // the host check says where
+    if (lp->h_flag[0] != 0 || lp->h_flag[1] != 0) FAIL(SCYLLA_ERR_INVALID_ARG, "malformed LP");  // the host check says where
   }
   if (host_tp) {
     CK(cudaMemcpyAsync(lp->t_rowptr, tp.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, st));

@@ -110,65 +110,48 @@ __global__ void k_column_kinds(long long n, const uint8_t* __restrict__ is_int, 
 //   (other_i |a_ij|) self_j on columns (the product order of the scaled values),
 // red = max for a Ruiz iteration and sum for the Pock-Chambolle step (alpha = 1);
 // a row without nonzeros keeps its factor.  The warp takes tiles t = first,
-// first + step, ...; a tile's indices and values come into shared memory with consecutive
-// lanes on consecutive entries, and the lanes of a row then walk its entries there, eight
-// gathers ahead.  The maximum compares bit patterns (the terms are not negative), on the
-// integer pipe: an FP64 maximum costs several instructions of the slow FP64 pipe.
-constexpr int kSetupTile = kTileNnz;
-struct SetupStage {
-  double val[kSetupTile];
-  int idx[kSetupTile];
-};
+// first + step, ...  The kernel is bound by the FP64 pipe (a warp instruction takes it
+// some 80 cycles; the square root and the division are about half of them), so the
+// maximum compares bit patterns (the terms are not negative) on the integer pipe, and a
+// column's maximum of (other a) self is that of other a, times self: rounding is
+// monotone.  The lanes of a row gather eight entries ahead.
+// (packing/covering 50k x 100k, 1M nonzeros, a Ruiz pass: 31.8 us with the tile's entries
+// staged in shared memory and the product per entry, 29.9 so; with the products formed by
+// consecutive lanes and reduced from shared memory, 39.0.)
 template <bool kMax, bool kRow>
 __device__ __forceinline__ void side_factor(int first, int step, const int2* __restrict__ tiles, int ntiles,
                                             const int* __restrict__ ptr, const int* __restrict__ idx,
                                             const double* __restrict__ vals, const double* __restrict__ self,
-                                            const double* __restrict__ other, double* __restrict__ out,
-                                            SetupStage& S) {
+                                            const double* __restrict__ other, double* __restrict__ out) {
   constexpr int kAhead = 8;
+  constexpr long long kInfBits = 0x7ff0000000000000LL;
+  constexpr bool kLater = kMax && !kRow;  // self multiplies the maximum
   const int lane = threadIdx.x & 31;
   for (int t = first; t < ntiles; t += step) {
-    const int2 ta = tiles[t], tb = tiles[t + 1];
-    const int nr = tb.x - ta.x, p0 = ta.y, n = tb.y - ta.y;
+    const int r0 = tiles[t].x, nr = tiles[t + 1].x - r0;
     const int sh = setup_row_lanes_log2(nr), L = 1 << sh, rl = lane >> sh, sub = lane & (L - 1);
-    const bool mine = rl < nr, staged = n <= kSetupTile;
-    const int row = ta.x + rl;
-    unsigned q0 = 0, q1 = 0;  // unsigned: a step past the longest row stays in range
-    double si = 0.0;
+    const bool mine = rl < nr;
+    const int row = r0 + rl;
+    unsigned p0 = 0, p1 = 0;  // unsigned: a step past the last entry stays in range
+    double si = 0.0, acc = 0.0;
+    long long top = 0;  // the bits of the maximum
     if (mine) {
-      q0 = unsigned(ptr[row] - p0);
-      q1 = unsigned(ptr[row + 1] - p0);
+      p0 = unsigned(ptr[row]) + sub;
+      p1 = unsigned(ptr[row + 1]);
       si = self[row];
     }
-    if (staged) {
-      __syncwarp();  // every lane is through with the last tile's entries
-#pragma unroll
-      for (int u = 0; u < kSetupTile / 32; ++u) {
-        const int q = lane + 32 * u;
-        if (q < n) {
-          S.idx[q] = idx[p0 + q];
-          S.val[q] = vals[p0 + q];
-        }
-      }
-      __syncwarp();
-    }
-    constexpr long long kInfBits = 0x7ff0000000000000LL;
-    double acc = 0.0;
-    long long top = 0;  // the bits of the maximum
-    for (unsigned q = q0 + sub; q < q1; q += kAhead * L) {
+    for (unsigned p = p0; p < p1; p += kAhead * L) {
       double a[kAhead], o[kAhead];
 #pragma unroll
-      for (int u = 0; u < kAhead; ++u) {
-        const unsigned e = q + u * L;
-        if (e < q1) {
-          o[u] = other[staged ? S.idx[e] : idx[p0 + e]];
-          a[u] = fabs(staged ? S.val[e] : vals[p0 + e]);
+      for (int u = 0; u < kAhead; ++u)
+        if (p + u * L < p1) {
+          o[u] = other[idx[p + u * L]];
+          a[u] = fabs(vals[p + u * L]);
         }
-      }
 #pragma unroll
       for (int u = 0; u < kAhead; ++u)
-        if (q + u * L < q1) {
-          const double term = kRow ? (si * a[u]) * o[u] : (o[u] * a[u]) * si;
+        if (p + u * L < p1) {
+          const double term = kRow ? (si * a[u]) * o[u] : (kLater ? o[u] * a[u] : (o[u] * a[u]) * si);
           const long long bits = __double_as_longlong(term);
           if (kMax) top = bits > top && bits <= kInfBits ? bits : top;  // a NaN is passed over, as by fmax
           else acc += term;
@@ -179,6 +162,7 @@ __device__ __forceinline__ void side_factor(int first, int step, const int2* __r
       else acc += __shfl_down_sync(0xffffffffu, acc, off);
     }
     if (kMax) acc = __longlong_as_double(top);
+    if (kLater) acc *= si;
     if (mine && sub == 0) out[row] = acc > 0.0 ? si / sqrt(acc) : si;
   }
 }
@@ -190,14 +174,13 @@ __global__ void __launch_bounds__(kSetupThreads) k_side_factors(DevSetup s, int 
                                                                const double* __restrict__ c, double* __restrict__ r2,
                                                                double* __restrict__ c2) {
   const int wpb = kSetupThreads / 32, w = int(threadIdx.x >> 5);
-  __shared__ SetupStage stage[kSetupThreads / 32];
   if (int(blockIdx.x) < gr) {
     side_factor<kMax, true>(int(blockIdx.x) * wpb + w, gr * wpb, s.a_tiles, s.a_ntiles, s.a_rowptr, s.a_cols,
-                            s.a_vals64, r, c, r2, stage[w]);
+                            s.a_vals64, r, c, r2);
   } else {
     const int b = int(blockIdx.x) - gr, gc = int(gridDim.x) - gr;
     side_factor<kMax, false>(b * wpb + w, gc * wpb, s.t_tiles, s.t_ntiles, s.t_rowptr, s.t_cols, s.t_vals64, c,
-                             r, c2, stage[w]);
+                             r, c2);
   }
 }
 
@@ -244,11 +227,20 @@ __global__ void __launch_bounds__(kSetupThreads)
                   const double* __restrict__ lo, const double* __restrict__ hi, long long m,
                   double* __restrict__ part) {
   const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
-  double mx = 0.0, s = 0.0, cs = 0.0, qs = 0.0;
-  for (long long p = t0; p < nnz; p += stride) {
-    const double v = a[p];
-    mx = fmax(mx, fabs(v));
-    s += v * v;
+  long long top = 0;  // the bits of the maximum, a NaN passed over
+  double s = 0.0, cs = 0.0, qs = 0.0;
+  constexpr int kAhead = 8;  // loads before the chain of additions
+  for (long long p = t0; p < nnz; p += kAhead * stride) {
+    double v[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) v[u] = p + u * stride < nnz ? a[p + u * stride] : 0.0;
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (p + u * stride < nnz) {
+        const long long bits = __double_as_longlong(v[u]) & 0x7fffffffffffffffLL;
+        top = bits > top && bits <= 0x7ff0000000000000LL ? bits : top;
+        s += v[u] * v[u];
+      }
   }
   for (long long j = t0; j < n; j += stride) cs += c[j] * c[j];
   for (long long i = t0; i < m; i += stride) {
@@ -256,18 +248,26 @@ __global__ void __launch_bounds__(kSetupThreads)
     const double q = fmax(x, y);
     qs += q * q;
   }
-  __shared__ double sh[4][kSetupThreads];
-  sh[0][threadIdx.x] = mx;
-  sh[1][threadIdx.x] = s;
-  sh[2][threadIdx.x] = cs;
-  sh[3][threadIdx.x] = qs;
+  // the three sums in thread order, each a chain of dependent additions, in a warp of its own
+  __shared__ double sh[3][kSetupThreads];
+  __shared__ long long tops[kSetupThreads / 32];
+  sh[0][threadIdx.x] = s;
+  sh[1][threadIdx.x] = cs;
+  sh[2][threadIdx.x] = qs;
+  for (int off = 16; off > 0; off >>= 1) top = max(top, __shfl_down_sync(0xffffffffu, top, off));
+  const int w = int(threadIdx.x >> 5);
+  if ((threadIdx.x & 31) == 0) tops[w] = top;
   __syncthreads();
-  if (threadIdx.x < 4) {
-    const int k = int(threadIdx.x);
-    double r = 0.0;
-    for (int q = 0; q < int(blockDim.x); ++q) r = k == 0 ? fmax(r, sh[0][q]) : r + sh[k][q];
-    part[4 * blockIdx.x + k] = r;
+  if ((threadIdx.x & 31) != 0 || w > 3) return;
+  double r = 0.0;
+  if (w < 3) {
+#pragma unroll 8
+    for (int q = 0; q < kSetupThreads; ++q) r += sh[w][q];
+  } else {
+    for (int q = 0; q < kSetupThreads / 32; ++q) top = max(top, tops[q]);
+    r = __longlong_as_double(top);
   }
+  part[4 * blockIdx.x + (w + 1) % 4] = r;
 }
 
 template <bool kMax>
@@ -280,7 +280,10 @@ void side_factors(const DevSetup& s, double* r, double* c, double* r2, double* c
 // names the place): column indices out of range or not increasing within a row, values or
 // costs not finite, bounds NaN, crossed or infinite on the wrong side, an integrality flag
 // other than 0 and 1, an integer column with a fractional finite bound.  rowptr is already
-// known to be non-decreasing from 0 to nnz.
+// known to be non-decreasing from 0 to nnz.  bad[0] is the flag; bad[1] counts the entries
+// that do not exceed the one before less those that start a row, which is 0 exactly when
+// every row increases (a search of rowptr at each such entry took 23.2 us instead of 11.4
+// on 50k rows and 1M nonzeros).
 __global__ void k_malformed(int m, int n, int nnz, const int* __restrict__ rowptr, const int* __restrict__ cols,
                             const double* __restrict__ vals, const double* __restrict__ c,
                             const double* __restrict__ lo, const double* __restrict__ hi, const double* __restrict__ l,
@@ -288,18 +291,15 @@ __global__ void k_malformed(int m, int n, int nnz, const int* __restrict__ rowpt
   const double inf = __longlong_as_double(0x7ff0000000000000LL);
   const long long stride = (long long)gridDim.x * blockDim.x, t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   bool w = false;
+  int falls = 0;  // entries whose column does not exceed the one before, less those that start a row
   for (long long p = t0; p < nnz; p += stride) {
     const int j = cols[p];
     w = w || j < 0 || j >= n || !isfinite(vals[p]);
-    if (p > 0 && cols[p - 1] >= j) {  // a row must start here: some rowptr entry is p
-      int a = 0, b = m;
-      while (a < b) {
-        const int mid = a + ((b - a) >> 1);
-        if (rowptr[mid] < p) a = mid + 1;
-        else b = mid;
-      }
-      w = w || rowptr[a] != p;
-    }
+    falls += p > 0 && cols[p - 1] >= j;
+  }
+  for (long long i = t0; i < m; i += stride) {
+    const int p = rowptr[i];
+    falls -= p > 0 && p < rowptr[i + 1] && cols[p - 1] >= cols[p];
   }
   auto bounds = [&](double a, double b) { return isnan(a) || isnan(b) || a > b || a == inf || b == -inf; };
   for (long long i = t0; i < m; i += stride) w = w || bounds(lo[i], hi[i]);
@@ -308,7 +308,9 @@ __global__ void k_malformed(int m, int n, int nnz, const int* __restrict__ rowpt
     w = w || !isfinite(c[j]) || bounds(l[j], u[j]) || k > 1 ||
         (k && ((isfinite(l[j]) && l[j] != floor(l[j])) || (isfinite(u[j]) && u[j] != floor(u[j]))));
   }
-  if (w) *bad = 1;
+  if (w) bad[0] = 1;
+  falls = __reduce_add_sync(0xffffffffu, falls);
+  if ((threadIdx.x & 31) == 0 && falls != 0) atomicAdd(bad + 1, falls);
 }
 
 }  // namespace
