@@ -33,7 +33,7 @@ CPP_SOURCES = ["lp.cpp", "fixprop.cpp", "pump.cpp", "batch.cpp", "fanout.cpp", "
 def _sources():
     return [os.path.join(CSRC, f) for f in CU_SOURCES + CPP_SOURCES] + \
         [os.path.join(CSRC, "internal.h"), os.path.join(CSRC, "lp_handle.h"), os.path.join(CSRC, "device_common.cuh"),
-         os.path.join(CSRC, "attempts.cuh"),
+         os.path.join(CSRC, "attempts.cuh"), os.path.join(CSRC, "conv_bits.h"),
          os.path.join(CSRC, "host_par.h"),
          os.path.join(INCLUDE, "scylla.h")]
 

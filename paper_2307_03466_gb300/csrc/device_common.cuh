@@ -11,6 +11,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "conv_bits.h"
 #include "internal.h"
 
 namespace scylla {
@@ -112,20 +113,21 @@ __device__ __forceinline__ void ld4_as(const V* p, V (&o)[4]) {
   else ld4(p, o);
 }
 
-// float -> double without the FP64 pipe (where a conversion costs as much as an FP64
-// add): sign, exponent rebiased by 1023 - 127, mantissa shifted into place; exact for
-// zeros and normal numbers, which is all the iterates hold; subnormals, infinities and
-// NaNs take the hardware conversion
+// conversions without the FP64 pipe (conv_bits.h)
 __device__ __forceinline__ double to_f64(float f) {
-  const unsigned int b = __float_as_uint(f);
-  const unsigned int e = (b >> 23) & 0xffu, man = b & 0x7fffffu;
-  if (e == 0xffu || (e == 0u && man != 0u)) return double(f);
-  const unsigned long long sign = (unsigned long long)(b >> 31) << 63;
-  const unsigned long long body =
-      e == 0u ? 0ULL : ((unsigned long long)(e + 896u) << 52) | ((unsigned long long)man << 29);
-  return __longlong_as_double((long long)(sign | body));
+  const bool small = fabsf(f) < 0x1p-100f;
+  return __longlong_as_double((long long)f64_bits(__float_as_uint(small ? f * 0x1p100f : f), small));
 }
 __device__ __forceinline__ double to_f64(double d) { return d; }
+__device__ __forceinline__ float to_f32(double d) {
+  return __uint_as_float(f32_bits((unsigned long long)__double_as_longlong(d)));
+}
+template <typename T>
+__device__ __forceinline__ T from_f64(double d);
+template <>
+__device__ __forceinline__ float from_f64<float>(double d) { return to_f32(d); }
+template <>
+__device__ __forceinline__ double from_f64<double>(double d) { return d; }
 
 __device__ __forceinline__ int skew(int q) { return q + (q >> 5); }
 
@@ -205,6 +207,16 @@ __device__ __forceinline__ double rc_proj(double r, double l, double u) {
   if (lf) return pos_bits(r) ? r : 0.0;
   if (uf) return neg_bits(r) ? r : 0.0;
   return 0.0;
+}
+
+__device__ __forceinline__ bool less_bits(double a, double b) {
+  return f64_less_bits(__double_as_longlong(a), __double_as_longlong(b));
+}
+
+// v - clamp(v, lo, hi): one subtraction, with 0 inside the bounds (a zero's sign is lost
+// in the squares it enters), and NaN for a NaN v
+__device__ __forceinline__ double beyond(double v, double lo, double hi) {
+  return v - (less_bits(v, lo) ? lo : (less_bits(hi, v) ? hi : v));
 }
 
 // The bound term of a multiplier v against a bound pair: a v when v > 0, b v when

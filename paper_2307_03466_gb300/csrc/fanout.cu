@@ -102,8 +102,8 @@ __device__ __forceinline__ void row_gather_pair(int p0, int p1, const int* __res
     if (p < p1) {
       cl = __ldg(cols + p);
       const double a = __ldg(vals + p);
-      hl = __double2float_rn(a);
-      ll = __double2float_rn(a - to_f64(hl));
+      hl = to_f32(a);
+      ll = to_f32(a - to_f64(hl));
     }
     const int cnt = p1 - b < 32 ? p1 - b : 32;
     for (int e = 0; e < cnt; e += 4) {
@@ -943,7 +943,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_fcheck_rows(DevFan<T> F) {
     const double ys[2] = {to_f64(y), to_f64(yav)};
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      const double rps = s[c] - clampv<double>(s[c], lo, hi);
+      const double rps = beyond(s[c], lo, hi);
       double* a = acc + 4 * c;
       a[0] += rps * rps;
       const double rp = rps * iRi;

@@ -1251,8 +1251,8 @@ struct CheckColsEpi {
       xav = blend(xav, x, w1, w);
       xa[j] = xav;
     }
-    aty_c[j] = T(s[0]);
-    aty_a[j] = T(s[1]);
+    aty_c[j] = from_f64<T>(s[0]);
+    aty_a[j] = from_f64<T>(s[1]);
     const double Cj = C[j], iCj = invC[j], cj = c64[j], lj = l64[j], uj = u64[j], xl = to_f64(eload<Coh>(xlr + j));
     const double xs[2] = {to_f64(x), to_f64(xav)};
     const bool has_q = QP == 1 || (QP == 2 && qq != nullptr);
@@ -1350,13 +1350,13 @@ struct CheckRowsEpi {
       yav = blend(yav, y, w1, w);
       ya[i] = yav;
     }
-    ax_c[i] = T(s[0]);
-    ax_a[i] = T(s[1]);
+    ax_c[i] = from_f64<T>(s[0]);
+    ax_a[i] = from_f64<T>(s[1]);
     const double iRi = invR[i], lo = lo64[i], hi = hi64[i], yl = to_f64(eload<Coh>(ylr + i));
     const double ys[2] = {to_f64(y), to_f64(yav)};
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-      const double rps = s[q] - clampv<double>(s[q], lo, hi);
+      const double rps = beyond(s[q], lo, hi);
       acc[4 * q + 0] += rps * rps;
       const double rp = rps * iRi;
       acc[4 * q + 1] += rp * rp;
