@@ -874,18 +874,22 @@ __global__ void __launch_bounds__(kFThreads, 3) k_fcheck_cols(DevFan<T> F) {
     const double cs = cc.at(int((F.lo_bits[j] >> k) & 1ULL) - int((F.up_bits[j] >> k) & 1ULL));
     const double xl = to_f64(F.XLR[o + k]);
     const double xs[2] = {to_f64(x), to_f64(xav)};
-    const bool boxed = above_neg_inf(lj) && below_pos_inf(uj);  // then r - lambda = 0 exactly
+    if (!(above_neg_inf(lj) && below_pos_inf(uj))) {  // otherwise r - lambda = 0 exactly
+      jump_over();
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const double r = cs - s[c];
+        const double rd = r - rc_proj(r, lj, uj);
+        acc[5 * c] += rd * rd;
+        const double rdu = rd * iCj;
+        acc[5 * c + 1] += rdu * rdu;
+      }
+    }
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       const double r = cs - s[c];
       const double lam = rc_proj(r, lj, uj);
       double* a = acc + 5 * c;
-      if (!boxed) {
-        const double rd = r - lam;
-        a[0] += rd * rd;
-        const double rdu = rd * iCj;
-        a[1] += rdu * rdu;
-      }
       a[2] += cs * xs[c];
       a[3] += bound_term(lam, lj, uj);
       const double dd = xs[c] - xl;

@@ -204,6 +204,13 @@ __device__ __forceinline__ bool spmv_tiles(const int2* __restrict__ tiles, int n
 #pragma unroll
       for (int it = 0; it < 3; ++it) {
         const int p = base + (it * 32 + lane) * kVec;
+        // FP64: the third step only holds the entries that the alignment left over
+        if constexpr (sizeof(Acc) == 8) {
+          if (it == 2) {
+            if (p >= p1) continue;
+            jump_over();
+          }
+        }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int q = p + e;
@@ -1253,25 +1260,30 @@ struct CheckColsEpi {
     }
     aty_c[j] = from_f64<T>(s[0]);
     aty_a[j] = from_f64<T>(s[1]);
-    const double Cj = C[j], iCj = invC[j], cj = c64[j], lj = l64[j], uj = u64[j], xl = to_f64(eload<Coh>(xlr + j));
+    const double cj = c64[j], lj = l64[j], uj = u64[j], xl = to_f64(eload<Coh>(xlr + j));
     const double xs[2] = {to_f64(x), to_f64(xav)};
     const bool has_q = QP == 1 || (QP == 2 && qq != nullptr);
     const double qj = has_q ? qq[j] : 0.0;
     // with both bounds finite the projection returns r itself, the dual residual
     // r - lambda is exactly 0 and its two squared norms are left as they are (the
     // same sums, without four FP64 instructions per iterate)
-    const bool boxed = above_neg_inf(lj) && below_pos_inf(uj);
+    if (!(above_neg_inf(lj) && below_pos_inf(uj))) {
+      jump_over();
+      const double iCj = invC[j];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const double r = has_q ? (cj + qj * xs[q]) - s[q] : cj - s[q];
+        const double rd = r - rc_proj(r, lj, uj);
+        acc[5 * q + 0] += rd * rd;
+        const double rdu = rd * iCj;
+        acc[5 * q + 1] += rdu * rdu;
+      }
+    }
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       // quadratic objective: reduced cost c + q x - A^T y; +-1/2 q x^2 in the objectives
       const double r = has_q ? (cj + qj * xs[q]) - s[q] : cj - s[q];
       const double lam = rc_proj(r, lj, uj);
-      if (!boxed) {
-        const double rd = r - lam;
-        acc[5 * q + 0] += rd * rd;
-        const double rdu = rd * iCj;
-        acc[5 * q + 1] += rdu * rdu;
-      }
       acc[5 * q + 2] += cj * xs[q];
       acc[5 * q + 3] += bound_term(lam, lj, uj);
       if (has_q) {
@@ -1282,7 +1294,7 @@ struct CheckColsEpi {
       const double dd = xs[q] - xl;
       acc[5 * q + 4] += dd * dd;
     }
-    if (hash_on && int_mask[j]) h += round_hash(j, xs[0] * Cj);
+    if (hash_on && int_mask[j]) h += round_hash(j, xs[0] * C[j]);
   }
 };
 
