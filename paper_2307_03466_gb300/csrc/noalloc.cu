@@ -117,10 +117,14 @@ __global__ void __launch_bounds__(kNaThreads) k_primal_residual_noalloc(
   }
   __shared__ double sh[kNaThreads / 32][kNaSums];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  {
+    // both sums in the association of na_warp_sum, each carried on by one half of the lanes:
+    // five additions a lane, not ten (each takes the FP64 pipe for 64 cycles a warp)
+    const bool hi = (lane & 16) != 0;
+    double t = (hi ? s[1] : s[0]) + __shfl_xor_sync(0xffffffffu, hi ? s[0] : s[1], 16);
 #pragma unroll
-  for (int k = 0; k < kNaSums; ++k) {
-    const double t = na_warp_sum(s[k]);
-    if (lane == 0) sh[w][k] = t;
+    for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((lane & 15) == 0) sh[w][lane >> 4] = t;
   }
   __syncthreads();
   if constexpr (!ONE) {
