@@ -137,7 +137,9 @@ typedef struct {
   int32_t autotune;             /* with prefetch = 0: 1 times the 32-row, wide-tile and (FP32) asynchronous-copy forms of the
                                    per-attempt kernels on the handle's own matrix at create and keeps the
                                    faster for each of the two kernels (the choice is kept per matrix shape
-                                   for the process); 0 takes the L2-size rule (1) */
+                                   for the process); 0 takes the L2-size rule.  A handle whose attempts run
+                                   resident (scylla_resident) launches neither kernel in a solve: it takes
+                                   the rule's form without timing (1) */
   int32_t infeasibility_checks; /* 1: at every check of a single-LP solve, test a candidate dual ray (the
                                    change of y since an earlier check) and end the solve SCYLLA_INFEASIBLE
                                    when it proves the LP infeasible (scylla_get_certificate); the
@@ -286,18 +288,19 @@ int scylla_time_kernels(scylla_lp* lp, int32_t attempts, double* ms);
  * staged, 5 asynchronous copies), the form the L2-size rule gives both, and the
  * create-time autotuner's device times per launch in ms, tune_ms[0..5] = primal and
  * dual of the 32-row form, of the wide form, and of the asynchronous-copy form (0
- * when it did not time them: a forced form, autotune = 0, FP64 for the last pair, or
- * the choice kept from an earlier handle of the same shape).  The autotuner picks
+ * when it did not time them: a forced form, autotune = 0, a handle whose attempts run
+ * resident, FP64 for the last pair, or the choice kept from an earlier handle of the same
+ * shape).  The autotuner picks
  * each kernel's form on its own.  Any output may be NULL. */
 int scylla_kernel_form(const scylla_lp* lp, int32_t* form, int32_t* form_dual, int32_t* rule_form,
                        double* tune_ms);
 
 /* Whether the handle's attempts run resident, all those between two checks in one
  * launch: *scope = 0 no (two launches per attempt), 1 in one cluster of *blocks blocks,
- * 2 in a cooperative grid of *blocks blocks.  Taken with use_graph = 1 and prefetch = 0
- * for LPs that the L2-size rule gives 32-row tiles and whose tiles fit the blocks' shared
- * memory; the results are those of the launched 32-row form bit for bit.  Either output
- * may be NULL. */
+ * 2 in a cooperative grid of *blocks blocks.  Taken with use_graph = 1 (or 3 where that
+ * runs as 1) and prefetch = 0 for LPs that the L2-size rule gives 32-row tiles and whose
+ * tiles fit the blocks' shared memory; the results are those of the launched 32-row form
+ * bit for bit.  Either output may be NULL. */
 int scylla_resident(const scylla_lp* lp, int32_t* scope, int32_t* blocks);
 
 /* Diagonal scaling A~ = diag(R) A diag(C) found at create: host, R length m_total,

@@ -789,13 +789,16 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
     CK(launch_init_point<double>(lp->d64, st));
   }
   CK(cudaStreamSynchronize(st));
-  // LPs that stay in L2 (the rule's 32-row plain form) run their attempts resident
-  // (attempts.cuh) and need no choice of a launched form
-  if (lp->p.prefetch == 0 && lp->form_rule == kFormPlain) {
+  // LPs that stay in L2 (the rule's 32-row plain form) run the chunk graphs' attempts
+  // resident (attempts.cuh) and need no choice of a launched form.  The other launch modes
+  // launch every attempt, so they keep the choice; use_graph = 3 runs chunk graphs where
+  // its persistent kernel does not take the solve.
+  const bool chunks = lp->p.use_graph == 1 || (lp->p.use_graph == 3 && (lp->p_grid <= 0 || lp->inf_cand));
+  if (lp->p.prefetch == 0 && lp->form_rule == kFormPlain && chunks) {
     ResidentPlan plan{};
     if (mixed ? resident_plan<float>(lp->d32, &plan) : resident_plan<double>(lp->d64, &plan)) {
       lp->tune = false;
-      if (lp->p.use_graph == 1) lp->resident = plan;
+      lp->resident = plan;
     }
   }
   if (lp->tune && later_w) {
