@@ -323,6 +323,7 @@ int create_batch(int32_t count, const scylla_csr* A, const double* const* c, con
   // tiles per LP, so none crosses an LP boundary
   std::vector<int2> at, tt;
   std::vector<int> alp, tlp, abeg(count + 1, 0), tbeg(count + 1, 0);
+  int longest = 0;
   for (int b = 0; b < count; ++b) {
     std::vector<int2> x = build_tiles_range(rp, h->row_off[b], h->row_off[b + 1]);
     abeg[b] = int(at.size());
@@ -336,6 +337,7 @@ int create_batch(int32_t count, const scylla_csr* A, const double* const* c, con
       tt.push_back(y[q]);
       tlp.push_back(b);
     }
+    longest = std::max(longest, int(std::max(x.size(), y.size())) - 1);
   }
   abeg[count] = int(at.size());
   tbeg[count] = int(tt.size());
@@ -530,6 +532,7 @@ int create_batch(int32_t count, const scylla_csr* A, const double* const* c, con
   };
   auto fill_b = [&](auto& B) {
     B.a_tile_lp = a_tlp; B.t_tile_lp = t_tlp; B.a_tile_beg = a_beg; B.t_tile_beg = t_beg;
+    B.longest = longest;
     B.ctl = ctl;
     B.tp_p = tp_p; B.tp_d = tp_d; B.tp_c1 = tp_c1; B.tp_c2 = tp_c2;
     B.n_done = n_done;

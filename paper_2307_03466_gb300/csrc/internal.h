@@ -169,6 +169,8 @@ struct DevBatch {
   long long* kglob;           // attempts made by the LPs still running
   double exp_red, exp_grow;
   int grid_p, grid_d, grid_c1, grid_c2;
+  int longest;                // most tiles of A^T or A of one LP
+  int ctl_warps;              // the control kernels take a warp per LP instead of a block
   int async_p, async_d;       // FP32: the primal / dual attempt kernel stages each warp's next tile by
                               // asynchronous copies
   int grid_pa, grid_da;       // their grids

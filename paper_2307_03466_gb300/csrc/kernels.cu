@@ -2314,11 +2314,21 @@ struct BDualEpi : DualEpi<T, Coh> {
   }
 };
 
-// A block per LP: its tiles' sums in lp_tile_sum's order, then the step decision (the
-// launch-per-phase path).  Warp 4 k + u takes the fourth u of sum k's running sums, so
-// the largest LP's chain is a twelfth of one warp's work and its loads come eight at a
-// time (64 LPs of up to 50k rows: 29 -> 9 us per attempt); the control block is decided on
-// in shared memory.
+// The launch-per-phase path's control kernels in two layouts with the same results.
+//
+// A block per LP: its tiles' sums in lp_tile_sum's order, then the step decision.  Warp
+// 4 k + u takes the fourth u of sum k's running sums, so the largest LP's chain is a
+// twelfth of one warp's work and its loads come eight at a time; the control block is
+// decided on in shared memory.
+//
+// A warp per LP, for many LPs: twelve warps each are mostly idle on small LPs, and past
+// one wave of blocks every wave costs what the first does.
+//
+// Per attempt, block / warp: 64 LPs of 60 rows 10.0 / 12.3 us, of 16,000 rows (1000 tiles)
+// 10.9 / 25.7; 512 LPs of 60 rows 14.4 / 13.3, of 4000 rows (250 tiles) 17.5 / 18.4; 1024
+// LPs of 60 rows 22.1 / 13.9, of 4000 28.5 / 18.5; 4096 LPs of 60 rows 63.4 / 29.0.  So
+// batch_grids takes blocks for what fits one wave of them and for fewer LPs than the
+// longest has tiles.  (Check control: 64 LPs 11.8 / 34.1 us, 1024 40 / 34, 4096 137 / 100.)
 constexpr int kBStepThreads = 12 * 32;
 template <typename T>
 __global__ void __launch_bounds__(kBStepThreads) k_bstep_control(DevBatch<T> B) {
@@ -2347,6 +2357,13 @@ __global__ void __launch_bounds__(kBStepThreads) k_bstep_control(DevBatch<T> B) 
     }
     ctl_out(B.ctl + b, &sc);
   }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_bstep_control_warps(DevBatch<T> B) {
+  const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (b >= B.nlp || !(B.slot[b].flags & kSlotActive)) return;
+  lp_step_decision<T>(&B, b, nullptr);
 }
 
 template <typename T>
@@ -2524,14 +2541,18 @@ __global__ void __launch_bounds__(kThreads) k_bcheck_rows(DevBatch<T> B) {
 // same attempt)
 constexpr int kBCheckThreads = (kNC1 + kNC2) * 32;
 template <typename T>
+__device__ __forceinline__ void batch_step_table(const DevBatch<T>& B) {
+  const long long k = *B.kglob;
+  for (int q = threadIdx.x; q < 2 * B.d.n_check; q += blockDim.x) {
+    const double kk = double(k + 1 + (q >> 1) + 1);
+    B.d.step_fac[q] = (q & 1) ? 1.0 + pow(kk, -B.exp_grow) : 1.0 - pow(kk, -B.exp_red);
+  }
+}
+template <typename T>
 __global__ void __launch_bounds__(kBCheckThreads) k_bcheck_control(DevBatch<T> B) {
   const int b = blockIdx.x;
   if (b == B.nlp) {
-    const long long k = *B.kglob;
-    for (int q = threadIdx.x; q < 2 * B.d.n_check; q += blockDim.x) {
-      const double kk = double(k + 1 + (q >> 1) + 1);
-      B.d.step_fac[q] = (q & 1) ? 1.0 + pow(kk, -B.exp_grow) : 1.0 - pow(kk, -B.exp_red);
-    }
+    batch_step_table(B);
     return;
   }
   if (!(B.slot[b].flags & kSlotCheck)) return;
@@ -2551,6 +2572,34 @@ __global__ void __launch_bounds__(kBCheckThreads) k_bcheck_control(DevBatch<T> B
   __syncwarp();
   check_control_warp(c, red, nullptr, 0);
   if (lane == 0) {
+    if (c->done) atomicAdd(B.n_done, 1);
+    write_slot(&B.slot[b], c);
+  }
+}
+// a warp per LP, the last block for the table
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_bcheck_control_warps(DevBatch<T> B) {
+  if (blockIdx.x == gridDim.x - 1) {
+    batch_step_table(B);
+    return;
+  }
+  const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (b >= B.nlp || !(B.slot[b].flags & kSlotCheck)) return;
+  double r[kNC1 + kNC2];
+#pragma unroll
+  for (int k = 0; k < kNC1 + kNC2; ++k) r[k] = 0.0;
+  for (int t = B.t_tile_beg[b] + lane; t < B.t_tile_beg[b + 1]; t += 32)
+#pragma unroll
+    for (int k = 0; k < kNC1; ++k) r[k] += B.tp_c1[kNC1 * t + k];
+  for (int t = B.a_tile_beg[b] + lane; t < B.a_tile_beg[b + 1]; t += 32)
+#pragma unroll
+    for (int k = 0; k < kNC2; ++k) r[kNC1 + k] += B.tp_c2[kNC2 * t + k];
+#pragma unroll
+  for (int k = 0; k < kNC1 + kNC2; ++k) r[k] = warp_sum(r[k]);
+  if (lane == 0) {
+    Control* c = &B.ctl[b];
+    c->k_fac = *B.kglob;
+    check_control(c, r, nullptr, 0);
     if (c->done) atomicAdd(B.n_done, 1);
     write_slot(&B.slot[b], c);
   }
@@ -3178,16 +3227,21 @@ static void batch_attempt_kernels(const DevBatch<double>& B, cudaStream_t st, in
   if (part != 0) k_bdual<double><<<B.grid_d, kThreads, 0, st>>>(B);
 }
 template <typename T>
+static void batch_step_kernel(const DevBatch<T>& B, cudaStream_t st) {
+  if (B.ctl_warps) k_bstep_control_warps<T><<<(B.nlp + kWarpsPerBlock - 1) / kWarpsPerBlock, kThreads, 0, st>>>(B);
+  else k_bstep_control<T><<<B.nlp, kBStepThreads, 0, st>>>(B);
+}
+template <typename T>
 cudaError_t launch_batch_slot(const DevBatch<T>& B, cudaStream_t st) {
   batch_attempt_kernels(B, st, -1);
-  k_bstep_control<T><<<B.nlp, kBStepThreads, 0, st>>>(B);
+  batch_step_kernel(B, st);
   return cudaGetLastError();
 }
 // one kernel of an attempt on its own (measurement): 0 primal, 1 dual, 2 step control
 template <typename T>
 cudaError_t launch_batch_part(const DevBatch<T>& B, int part, cudaStream_t st) {
   if (part == 0 || part == 1) batch_attempt_kernels(B, st, part);
-  else k_bstep_control<T><<<B.nlp, kBStepThreads, 0, st>>>(B);
+  else batch_step_kernel(B, st);
   return cudaGetLastError();
 }
 
@@ -3195,7 +3249,9 @@ template <typename T>
 cudaError_t launch_batch_check(const DevBatch<T>& B, cudaStream_t st) {
   k_bcheck_cols<T><<<B.grid_c1, kThreads, 0, st>>>(B);
   k_bcheck_rows<T><<<B.grid_c2, kThreads, 0, st>>>(B);
-  k_bcheck_control<T><<<B.nlp + 1, kBCheckThreads, 0, st>>>(B);
+  if (B.ctl_warps)
+    k_bcheck_control_warps<T><<<(B.nlp + kWarpsPerBlock - 1) / kWarpsPerBlock + 1, kThreads, 0, st>>>(B);
+  else k_bcheck_control<T><<<B.nlp + 1, kBCheckThreads, 0, st>>>(B);
   return cudaGetLastError();
 }
 template <typename T>
@@ -3252,26 +3308,29 @@ cudaError_t launch_batch_compact(const DevBatch<T>& B, cudaStream_t st) {
 
 template <typename T>
 void batch_grids(DevBatch<T>& B) {
-  auto grid = [](const void* k, int tiles, size_t smem) {
+  auto wave = [](const void* k, int threads) {
     int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads, smem) != cudaSuccess || per_sm < 1)
-      per_sm = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
+    return (long long)per_sm * device_sm_count();
+  };
+  auto grid = [&](const void* k, int tiles) {
     long long need = tiles;  // a whole wave, or one block per tile (as occupancy_grid)
     if (need < 1) need = 1;
-    const long long cap = (long long)per_sm * device_sm_count();
+    const long long cap = wave(k, kThreads);
     return int(need < cap ? need : cap);
   };
-  B.grid_p = grid((const void*)k_bprimal<T>, B.d.t_ntiles, 0);
-  B.grid_d = grid((const void*)k_bdual<T>, B.d.a_ntiles, 0);
+  B.ctl_warps = B.nlp > wave((const void*)k_bstep_control<T>, kBStepThreads) && B.nlp > B.longest ? 1 : 0;
+  B.grid_p = grid((const void*)k_bprimal<T>, B.d.t_ntiles);
+  B.grid_d = grid((const void*)k_bdual<T>, B.d.a_ntiles);
   if constexpr (std::is_same<T, float>::value) {
-    B.grid_pa = grid((const void*)k_bprimal_as, B.d.t_ntiles, 0);
-    B.grid_da = grid((const void*)k_bdual_as, B.d.a_ntiles, 0);
+    B.grid_pa = grid((const void*)k_bprimal_as, B.d.t_ntiles);
+    B.grid_da = grid((const void*)k_bdual_as, B.d.a_ntiles);
   } else {
     B.grid_pa = B.grid_p;
     B.grid_da = B.grid_d;
   }
-  B.grid_c1 = grid((const void*)k_bcheck_cols<T>, B.d.t_ntiles, 0);
-  B.grid_c2 = grid((const void*)k_bcheck_rows<T>, B.d.a_ntiles, 0);
+  B.grid_c1 = grid((const void*)k_bcheck_cols<T>, B.d.t_ntiles);
+  B.grid_c2 = grid((const void*)k_bcheck_rows<T>, B.d.a_ntiles);
 }
 
 #define SCYLLA_INSTANTIATE_BATCH(T)                                                                   \
