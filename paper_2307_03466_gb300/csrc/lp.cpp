@@ -406,27 +406,34 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
   lp->nnz0 = nnz0;
   // the l2 distance needs no auxiliary columns
   const bool aux_on = lp->p.aux_general_integers != 0 && lp->p.distance == 1;
+  // slices of n for the host threads
+  const int slices = int(std::max<int64_t>(1, std::min<int64_t>(64, n0 / 65536)));
   {
     int64_t k = 0;
     for (int64_t j = 0; j < n0; ++j) k += is_int[j] != 0;
     lp->n_int = k;
     lp->gen_int.clear();
-    if (aux_on && k > 0)
-      for (int64_t j = 0; j < n0; ++j)
-        if (is_int[j] && u[j] - l[j] != 1.0) lp->gen_int.push_back(int32_t(j));
+    if (aux_on && k > 0) {
+      // (one thread took 1.8 ms longer on a million columns, a tenth of the call)
+      std::vector<std::vector<int32_t>> gen(static_cast<size_t>(slices));
+      fork_join(slices, [&](int t) {
+        for (int64_t j = n0 * t / slices; j < n0 * (t + 1) / slices; ++j)
+          if (is_int[j] && u[j] - l[j] != 1.0) gen[size_t(t)].push_back(int32_t(j));
+      });
+      for (const auto& g : gen) lp->gen_int.insert(lp->gen_int.end(), g.begin(), g.end());
+    }
   }
-  // ||c||: in chunks fixed by n, each in order, so that it does not depend on the host's
+  // ||c||: in slices fixed by n, each in order, so that it does not depend on the host's
   // thread count
   auto c_norm = [&] {
-    const int chunks = int(std::max<int64_t>(1, std::min<int64_t>(64, n0 / 65536)));
-    std::vector<double> c2(size_t(chunks), 0.0);
-    fork_join(chunks, [&](int t) {
+    std::vector<double> c2(size_t(slices), 0.0);
+    fork_join(slices, [&](int t) {
       double s2 = 0.0;
-      for (int64_t j = n0 * t / chunks; j < n0 * (t + 1) / chunks; ++j) s2 += c[j] * c[j];
+      for (int64_t j = n0 * t / slices; j < n0 * (t + 1) / slices; ++j) s2 += c[j] * c[j];
       c2[size_t(t)] = s2;
     });
     double s2 = 0.0;
-    for (int t = 0; t < chunks; ++t) s2 += c2[size_t(t)];
+    for (int t = 0; t < slices; ++t) s2 += c2[size_t(t)];
     return std::sqrt(s2);
   };
   const int64_t na = int64_t(lp->gen_int.size());
@@ -446,8 +453,13 @@ static int create_impl(const scylla_csr* A, const double* c, const double* lo, c
   if (na > 0) {
     ci_aux.resize(nnz);
     va_aux.resize(nnz);
-    std::copy(A->cols, A->cols + nnz0, ci_aux.begin());
-    std::copy(A->vals, A->vals + nnz0, va_aux.begin());
+    // (no host pass has read these arrays before, where the device validates them)
+    const int pieces = int(std::max<int64_t>(1, std::min<int64_t>(64, nnz0 / 262144)));
+    fork_join(pieces, [&](int t) {
+      const int64_t b = nnz0 * t / pieces, e = nnz0 * (t + 1) / pieces;
+      std::copy(A->cols + b, A->cols + e, ci_aux.begin() + b);
+      std::copy(A->vals + b, A->vals + e, va_aux.begin() + b);
+    });
     for (int64_t t = 0; t < na; ++t) {
       const int j = lp->gen_int[t];
       const int64_t r0 = m0 + 2 * t, p = nnz0 + 4 * t;
