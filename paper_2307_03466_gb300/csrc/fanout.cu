@@ -451,6 +451,18 @@ __device__ __forceinline__ void fan_block_sums(A (&acc)[NSUM][FanGeo<VEC, CHUNK>
   }
 }
 
+// Whether an attempt's dual step, or a check's row half, has an objective to work on.
+// The kernel after it (and the copies after that one) takes the answer from the state:
+// the control kernels count finished objectives themselves, so a block of theirs that
+// looked at the count could find it changed by its own launch and skip its duties (the
+// attempt's count, an earlier flag's reset).
+template <typename T>
+__device__ __forceinline__ bool fan_live(const DevFan<T>& F) {
+  const bool live = *F.n_done < F.K;
+  if (blockIdx.x == 0 && threadIdx.x == 0) F.state->live = live ? 1 : 0;
+  return live;
+}
+
 // Primal SpMM of one attempt for every objective (Algorithm 1, primal step):
 // x'_jk = proj_[l_j,u_j](x_jk + tau_k ((A^T Y)_jk - c_hat_jk)), the running average
 // and ||x' - x||^2 per objective.  Row groups are dealt gw, gw + nw, ...; while a
@@ -589,7 +601,7 @@ template <typename T, int VEC, int CHUNK>
 __global__ void __launch_bounds__(kFThreads, sizeof(T) == 4 && !(VEC == 4 && CHUNK == 32) ? 4 : 3) k_fdual(DevFan<T> F) {
   typedef typename AccOf<T>::type A;
   typedef FanGeo<VEC, CHUNK> G;
-  if (*F.n_done >= F.K) return;
+  if (!fan_live(F)) return;
   __shared__ double sh[kFWarps * 2 * kFK];
   __shared__ __align__(16) FanShared<T> S;
   __shared__ __align__(16) FanStage<T, VEC> E;
@@ -756,8 +768,8 @@ __device__ __forceinline__ void write_fan_slot(FanSlot<T>* s, const Control* c) 
 constexpr int kFStepThreads = 3 * 32;
 template <typename T>
 __global__ void __launch_bounds__(kFStepThreads) k_fstep_control(DevFan<T> F) {
-  if (*F.n_done >= F.K) return;  // nothing attempted: the pools keep their roles
   FanState* st = F.state;
+  if (!st->live) return;  // nothing attempted: the pools keep their roles
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ++*F.kglob;
     ++st->att;
@@ -904,7 +916,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_fcheck_cols(DevFan<T> F) {
 // Row half of a check, laid out as the column half.
 template <typename T>
 __global__ void __launch_bounds__(kFThreads, 3) k_fcheck_rows(DevFan<T> F) {
-  if (*F.n_done >= F.K) return;
+  if (!fan_live(F)) return;
   __shared__ double sh[kFWarps * kNC2 * 32];
   const int lane = threadIdx.x & 31, halves = fan_halves(F.K);
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
@@ -968,8 +980,8 @@ __global__ void __launch_bounds__(kFThreads, 3) k_fcheck_rows(DevFan<T> F) {
 constexpr int kFCheckThreads = (kNC1 + kNC2) * 32;
 template <typename T>
 __global__ void __launch_bounds__(kFCheckThreads) k_fcheck_control(DevFan<T> F) {
-  if (*F.n_done >= F.K) return;
   FanState* st = F.state;
+  if (!st->live) return;
   const long long k0 = *F.kglob;
   constexpr bool f32 = sizeof(T) == 4;
   const int k = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1038,9 +1050,8 @@ __global__ void __launch_bounds__(kFCheckThreads) k_fcheck_control(DevFan<T> F) 
 // per (row, flagged objective) pair; nothing to do unless a flag is set.
 template <typename T, bool RST>
 __global__ void __launch_bounds__(kFThreads) k_fcopy(DevFan<T> F) {
-  // every objective finished: no attempt was made, the flags are an earlier one's
-  if (!RST && *F.n_done >= F.K) return;
   const FanState* st = F.state;
+  if (!st->live) return;  // no attempt or check was made: the flags are an earlier one's
   const unsigned char* flag = RST ? st->rst : st->rej;
   // the flagged objectives, ascending
   __shared__ int list[kFK];
