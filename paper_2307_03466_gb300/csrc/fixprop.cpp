@@ -371,7 +371,10 @@ namespace {
 // The integer columns by (distance of xbar to its rounding, index).  At an LP point most
 // distances are exactly 0: those columns come first, in index order, and only the others
 // are sorted, as (distance, index) pairs (packing/covering 8000 x 20,000 with 8000 binaries:
-// the comparisons through an index array had been a third of the call).
+// the comparisons through an index array had been a third of the call).  The pairs come in
+// index order and many distances are equal, so the sort is a stable one by the distance
+// (62,500 columns at two distances 1.2 ms, by an unstable one of the pairs 3.6; at random
+// ones 5.4 and 6.5).
 std::vector<int32_t> fixing_order(const scylla_lp& lp, const double* xbar) {
   std::vector<int32_t> order;
   order.reserve(size_t(lp.n_int));
@@ -384,17 +387,17 @@ std::vector<int32_t> fixing_order(const scylla_lp& lp, const double* xbar) {
     if (d == 0.0) order.push_back(int32_t(j));
     else rest.emplace_back(d, int32_t(j));
   }
-  auto before = [](const std::pair<double, int32_t>& a, const std::pair<double, int32_t>& b) {
-    return a.first != b.first ? a.first < b.first : a.second < b.second;
-  };
+  typedef std::pair<double, int32_t> Dist;
   if (finite) {
-    std::sort(rest.begin(), rest.end(), before);
+    std::stable_sort(rest.begin(), rest.end(), [](const Dist& a, const Dist& b) { return a.first < b.first; });
   } else {
     // an infinite entry has no distance: the order of the comparison sort over every column
-    std::vector<std::pair<double, int32_t>> all;
+    std::vector<Dist> all;
     for (int64_t j = 0; j < lp.n0; ++j)
       if (lp.int0[j]) all.emplace_back(std::fabs(xbar[j] - round_half_up(xbar[j])), int32_t(j));
-    std::stable_sort(all.begin(), all.end(), before);
+    std::stable_sort(all.begin(), all.end(), [](const Dist& a, const Dist& b) {
+      return a.first != b.first ? a.first < b.first : a.second < b.second;
+    });
     order.clear();
     rest.swap(all);
   }
