@@ -414,7 +414,10 @@ void fix_one(const scylla_lp& lp, const RootState& root, const double* xbar, dou
   int64_t nf = 0;
   for (size_t k = 0; k < order.size(); ++k) {
     const int64_t j = order[k];
-    if (k + 2 < order.size()) pr.prefetch(order[k + 2]);
+    if (k + 2 < order.size()) {
+      const Propagator::Dom& d2 = pr.dom[size_t(order[k + 2])];
+      if (d2.lb != d2.ub) pr.prefetch(order[k + 2]);  // the propagation fixes most columns of an assignment
+    }
     Propagator::Dom& d = pr.dom[size_t(j)];
     if (d.lb == d.ub) continue;
     double v = round_half_up(xbar[j]);
