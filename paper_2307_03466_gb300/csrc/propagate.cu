@@ -48,14 +48,21 @@ __global__ void k_prop_perm(int n, const int* __restrict__ t_rowptr, const int* 
   }
 }
 
-// the caller's domains side by side, and whether an integer column's is fractional (then
-// no row is screened: the rounding alone changes such a bound)
-__global__ void k_prop_in(PropDev P) {
+// The start of a call: the caller's domains side by side, and whether an integer column's
+// is fractional (then no row is screened: the rounding alone changes such a bound); no
+// column has a proposal, no row is ignored, every row is active.
+__global__ void k_prop_in(PropDev P, unsigned char* __restrict__ active) {
   bool frac = false;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < P.n; j += gridDim.x * blockDim.x) {
+  const int t0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+  for (int j = t0; j < P.n; j += stride) {
     const double l = P.dl[j], u = P.du[j];
     P.dom[j] = make_double2(l, u);
+    P.flag[j] = 0;
     frac = frac || (P.is_int[j] && (l != floor(l) || u != floor(u)));
+  }
+  for (int i = t0; i < P.m; i += stride) {
+    P.state[i] = 0;
+    active[i] = 1;
   }
   if (frac) P.ctl->fractional = 1;
 }
@@ -241,12 +248,9 @@ cudaError_t propagate_perm(int n, const int* t_rowptr, const int* t_rows, const 
 }
 
 cudaError_t propagate_start(const PropDev& P, unsigned char* active, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(P.ctl, 0, sizeof(PropCtl), st);
-  if (e == cudaSuccess && P.m > 0) e = cudaMemsetAsync(P.state, 0, size_t(P.m), st);
-  if (e == cudaSuccess && P.m > 0) e = cudaMemsetAsync(active, 1, size_t(P.m), st);
-  if (e == cudaSuccess && P.n > 0) e = cudaMemsetAsync(P.flag, 0, size_t(P.n), st);
+  const cudaError_t e = cudaMemsetAsync(P.ctl, 0, sizeof(PropCtl), st);
   if (e != cudaSuccess) return e;
-  if (P.n > 0) k_prop_in<<<prop_grid(P.n), kPropThreads, 0, st>>>(P);
+  k_prop_in<<<prop_grid(P.m > P.n ? P.m : P.n), kPropThreads, 0, st>>>(P, active);
   return cudaGetLastError();
 }
 
