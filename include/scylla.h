@@ -300,7 +300,14 @@ int scylla_kernel_form(const scylla_lp* lp, int32_t* form, int32_t* form_dual, i
  * 2 in a cooperative grid of *blocks blocks.  Taken with use_graph = 1 (or 3 where that
  * runs as 1) and prefetch = 0 for LPs that the L2-size rule gives 32-row tiles and whose
  * tiles fit the blocks' shared memory; the results are those of the launched 32-row form
- * bit for bit.  Either output may be NULL. */
+ * bit for bit.  The grid has one block per SM and keeps every SM for up to n_check
+ * attempts, so other kernels on the device (of other streams or processes) start after it
+ * instead of beside it; while another solve of this process is under way on the device
+ * (also of a batch or a fan-out), a handle with scope 2 launches its attempts one by one,
+ * chunk by chunk, and prefetch = 4 makes a handle do so always.  A wait at the grid's
+ * barrier is bounded by device_wait_limit_s: a kernel of another stream that holds SMs for
+ * longer than that while the grid starts ends the solve with SCYLLA_ERR_TIMEOUT.  Either
+ * output may be NULL. */
 int scylla_resident(const scylla_lp* lp, int32_t* scope, int32_t* blocks);
 
 /* Diagonal scaling A~ = diag(R) A diag(C) found at create: host, R length m_total,

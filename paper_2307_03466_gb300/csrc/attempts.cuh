@@ -28,7 +28,6 @@
 // order.
 #pragma once
 
-constexpr int kScopeCluster = 1, kScopeGrid = 2;
 constexpr int kResTile = kTileNnz;  // entries of a tile's slot in shared memory
 constexpr int kResMaxPart = 512;    // tiles of a side in the cluster scope
 constexpr int kResMaxVb = 8;        // virtual blocks per block in the grid scope

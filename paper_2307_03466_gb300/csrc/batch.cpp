@@ -36,6 +36,7 @@ struct scylla_batch {
   cudaEvent_t ev_chunk[2] = {nullptr, nullptr};
   int* h_done = nullptr;  // pinned, two slots
   double* h_io = nullptr;  // pinned, kReadStage doubles behind h_done (read_back)
+  int device = 0;
   int nlp = 0;
   std::vector<int> row_off, col_off;  // per LP (nlp + 1)
   int m = 0, n = 0, nnz = 0;
@@ -259,6 +260,7 @@ int create_batch(int32_t count, const scylla_csr* A, const double* const* c, con
   const bool mixed = h->p.precision == SCYLLA_PREC_MIXED;
   h->nlp = count;
   h->user_st = static_cast<cudaStream_t>(stream);
+  CKB(cudaGetDevice(&h->device));
   CKB(cudaStreamCreateWithFlags(&h->st, cudaStreamNonBlocking));
   for (cudaEvent_t* e : {&h->ev_user, &h->ev0, &h->ev1}) CKB(cudaEventCreate(e));
   for (int k = 0; k < 2; ++k) CKB(cudaEventCreateWithFlags(&h->ev_chunk[k], cudaEventDisableTiming));
@@ -683,6 +685,7 @@ extern "C" int scylla_batch_solve(scylla_batch* h, double tol, int64_t iter_limi
     set_error("need tol >= 0 and iter_limit >= 0");
     return SCYLLA_ERR_INVALID_ARG;
   }
+  const SolveUnderWay busy(h->device);
   if (h->user_st) {
     CKB(cudaEventRecord(h->ev_user, h->user_st));
     CKB(cudaStreamWaitEvent(h->st, h->ev_user, 0));

@@ -428,6 +428,7 @@ extern "C" int scylla_fanout_solve(scylla_fanout* f, double tol, int64_t iter_li
     set_error("invalid argument");
     return SCYLLA_ERR_INVALID_ARG;
   }
+  const SolveUnderWay busy(f->lp->device);
   const bool mixed = f->lp->p.precision == SCYLLA_PREC_MIXED;
   const int rc = mixed ? fan_solve_impl<float>(f, f->f32, tol, iter_limit)
                        : fan_solve_impl<double>(f, f->f64, tol, iter_limit);

@@ -422,8 +422,9 @@ cudaError_t launch_persistent(const DevLP<T>& d, void* grid_bar, int grid, doubl
 // the resident form of the per-attempt kernels (attempts.cuh): its launch for an LP
 // (false when it cannot run), and the launch of up to n_check attempts; bar:
 // kGridBarBytes
+constexpr int kScopeCluster = 1, kScopeGrid = 2;
 struct ResidentPlan {
-  int scope;             // 0 none, 1 a cluster of blocks, 2 a grid of one block per SM
+  int scope;             // 0 none, a cluster of blocks, a grid of one block per SM
   int blocks, threads;
   int tpw;               // most tiles of a side per warp
   int slots_t, slots_a;  // tile slots per block in shared memory, of the transpose and of A
@@ -433,6 +434,24 @@ template <typename T>
 bool resident_plan(const DevLP<T>& d, ResidentPlan* out);
 template <typename T>
 cudaError_t launch_attempts(const DevLP<T>& d, const ResidentPlan& p, void* bar, cudaStream_t st);
+// A solve of this process under way on a device, for as long as the object lives.  The grid
+// scope of the resident form takes every SM for a chunk, so a solve takes it only while it
+// is alone; beside others it launches its attempts, which share the SMs (the results are the
+// same bit for bit).  2000 attempts of each of T handles at once, always resident / by this
+// rule: knapsack LP of 5000 rows, FP32-mixed, T = 1 16.1 / 16.1 ms, 2 31.0 / 26.6, 4 61.1 /
+// 36.0, 8 122 / 66.5; packing/covering 50k x 100k, FP64, 64.0 / 64.0, 127 / 117, 254 / 212,
+// 509 / 440.
+class SolveUnderWay {
+ public:
+  explicit SolveUnderWay(int device);
+  ~SolveUnderWay();
+  SolveUnderWay(const SolveUnderWay&) = delete;
+  SolveUnderWay& operator=(const SolveUnderWay&) = delete;
+  static bool alone(int device);  // at most one solve is under way
+
+ private:
+  int device_;
+};
 constexpr int kPersistentPartials = 24;  // doubles per block in DevLP::pp_part
 constexpr size_t kGridBarBytes = 16;
 template <typename T>

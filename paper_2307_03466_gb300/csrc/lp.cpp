@@ -6,6 +6,7 @@
 // whose device-side while loop runs until the device control block says done.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -918,6 +919,10 @@ void scylla_lp::drop_graphs() {
   if (chunk_graph) cudaGraphDestroy(chunk_graph);
   chunk_exec = nullptr;
   chunk_graph = nullptr;
+  if (shared_exec) cudaGraphExecDestroy(shared_exec);
+  if (shared_graph) cudaGraphDestroy(shared_graph);
+  shared_exec = nullptr;
+  shared_graph = nullptr;
 }
 
 void scylla_lp::set_qp_active(bool on) {
@@ -1077,12 +1082,14 @@ static int build_graph(scylla_lp* lp, const DevLP<T>& d) {
   return rc;
 }
 
+// n_check attempts (resident or launched) and a check
 template <typename T>
-static int build_chunk_graph(scylla_lp* lp, const DevLP<T>& d) {
+static int build_chunk_graph(scylla_lp* lp, const DevLP<T>& d, bool resident, cudaGraph_t* graph,
+                             cudaGraphExec_t* graph_exec) {
   cudaStream_t st = lp->st;
   CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
-  if (lp->resident.scope) {
+  if (resident) {
     e = launch_attempts<T>(d, lp->resident, lp->grid_bar, st);
     if (e == cudaSuccess) e = launch_check<T>(d, st, false);
   } else {
@@ -1102,10 +1109,18 @@ static int build_chunk_graph(scylla_lp* lp, const DevLP<T>& d) {
     cudaGraphDestroy(g);
     CK(e3);
   }
-  lp->chunk_graph = g;
-  lp->chunk_exec = exec;
+  *graph = g;
+  *graph_exec = exec;
   return SCYLLA_OK;
 }
+
+namespace scylla {
+static std::atomic<int> g_under_way[64];  // by device
+static std::atomic<int>& under_way(int device) { return g_under_way[std::min(std::max(device, 0), 63)]; }
+SolveUnderWay::SolveUnderWay(int device) : device_(device) { ++under_way(device_); }
+SolveUnderWay::~SolveUnderWay() { --under_way(device_); }
+bool SolveUnderWay::alone(int device) { return under_way(device).load() <= 1; }
+}  // namespace scylla
 
 template <typename T>
 static int solve_impl(scylla_lp* lp, const DevLP<T>& d, double tol, int64_t iter_limit, int stall_checks) {
@@ -1139,28 +1154,31 @@ static int solve_impl(scylla_lp* lp, const DevLP<T>& d, double tol, int64_t iter
     CK(cudaGraphLaunch(lp->exec, st));
     launches = -1;  // counted on the device
   } else if (lp->p.use_graph == 1 || lp->p.use_graph == 3) {
-    if (!lp->chunk_exec) {
-      const int rc = build_chunk_graph<T>(lp, d);
-      if (rc != SCYLLA_OK) return rc;
-    }
     // chunk c+1 is queued before the done flag of chunk c is read, so the GPU never
     // waits for the host; the chunk queued after the last one returns at once.  A chunk's
     // whole control block comes back, so that a solve whose last chunk has no successor
     // ends with that copy and its event.
-    auto enqueue = [&](long long c) -> cudaError_t {
-      cudaError_t e = cudaGraphLaunch(lp->chunk_exec, st);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&lp->h_chunk[c & 1], lp->ctl, sizeof(Control), cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaEventRecord(lp->ev_chunk[c & 1], st);
+    auto enqueue = [&](long long c) -> int {
+      const bool share = lp->resident.scope == kScopeGrid && !SolveUnderWay::alone(lp->device);
+      cudaGraphExec_t& exec = share ? lp->shared_exec : lp->chunk_exec;
+      if (!exec) {
+        const int rc = build_chunk_graph<T>(lp, d, !share && lp->resident.scope != 0,
+                                            share ? &lp->shared_graph : &lp->chunk_graph, &exec);
+        if (rc != SCYLLA_OK) return rc;
+      }
+      CK(cudaGraphLaunch(exec, st));
+      CK(cudaMemcpyAsync(&lp->h_chunk[c & 1], lp->ctl, sizeof(Control), cudaMemcpyDeviceToHost, st));
+      CK(cudaEventRecord(lp->ev_chunk[c & 1], st));
       launches += per_chunk;
-      return e;
+      return SCYLLA_OK;
     };
     // the check at the iteration limit ends the solve, so no chunk is queued ahead past it
     const long long need = (iter_limit + nchk - 1) / nchk;
-    CK(enqueue(0));
-    for (long long c = 0; c < max_chunks; ++c) {
+    int rc = enqueue(0);
+    for (long long c = 0; rc == SCYLLA_OK && c < max_chunks; ++c) {
       const bool ahead = c + 1 < need;
-      if (ahead) CK(enqueue(c + 1));
+      if (ahead) rc = enqueue(c + 1);
+      if (rc != SCYLLA_OK) break;
       CK(cudaEventSynchronize(lp->ev_chunk[c & 1]));
       if (lp->h_chunk[c & 1].done) {
         if (ahead) break;
@@ -1169,8 +1187,9 @@ static int solve_impl(scylla_lp* lp, const DevLP<T>& d, double tol, int64_t iter
         lp->last_launches = launches;
         return SCYLLA_OK;
       }
-      if (!ahead && c + 1 < max_chunks) CK(enqueue(c + 1));
+      if (!ahead && c + 1 < max_chunks) rc = enqueue(c + 1);
     }
+    if (rc != SCYLLA_OK) return rc;
   } else {
     for (long long ch = 0; ch < max_chunks; ++ch) {
       CK(cudaMemcpyAsync(lp->h_ctl, lp->ctl, sizeof(Control), cudaMemcpyDeviceToHost, st));
@@ -1189,6 +1208,7 @@ static int solve_impl(scylla_lp* lp, const DevLP<T>& d, double tol, int64_t iter
 }
 
 int scylla_lp::solve(double tol, int64_t iter_limit, int stall_checks, scylla_pdhg_result* out) {
+  const SolveUnderWay busy(device);
   int rc = order_after_user();
   if (rc != SCYLLA_OK) return rc;
   rc = (p.precision == SCYLLA_PREC_MIXED) ? solve_impl<float>(this, d32, tol, iter_limit, stall_checks)

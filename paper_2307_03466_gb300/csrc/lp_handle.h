@@ -113,6 +113,8 @@ struct scylla_lp {
   cudaGraphConditionalHandle cond = 0;
   cudaGraph_t chunk_graph = nullptr;  // n_check attempts + one check (use_graph = 1)
   cudaGraphExec_t chunk_exec = nullptr;
+  cudaGraph_t shared_graph = nullptr;  // the same with launched attempts, of a handle whose
+  cudaGraphExec_t shared_exec = nullptr;  // attempts run resident in the grid scope (SolveUnderWay)
   cudaEvent_t ev_chunk[2] = {nullptr, nullptr};
   scylla::Control* h_chunk = nullptr;  // pinned: the control block after a chunk, two slots
   int* h_flag = nullptr;               // pinned
