@@ -491,10 +491,10 @@ int scylla_get_trace(const scylla_lp* lp, double* steps, int64_t* n_steps, doubl
  * the array's device address up (cudaGetSymbolAddress, with that device current)
  * and keeps it for the life of the process, so make that first call before any
  * stream capture, and do not use the entry point across a cudaDeviceReset (the kept
- * address would be stale).  Every call clears the array's arrival counter on its
- * stream (cudaMemsetAsync) before its kernel, so a call that failed part way leaves
- * nothing behind for the next one.  Every call shares the array, so calls that
- * overlap on the GPU race and must be serialised by the caller.  Nothing is
+ * address would be stale).  A call of more than 256 rows (one block) clears the array's
+ * arrival counter on its stream (cudaMemsetAsync) before its kernel, so a call that
+ * failed part way leaves nothing behind for the next one.  Such calls share the array, so
+ * those that overlap on the GPU race and must be serialised by the caller.  Nothing is
  * allocated, by this library or by any library it calls.
  * Errors: INVALID_ARG (sizes, null pointers), UNSUPPORTED (device ordinal >= 64),
  * CUDA. */

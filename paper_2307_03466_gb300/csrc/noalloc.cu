@@ -45,13 +45,13 @@ __device__ __forceinline__ double na_warp_sum(double v) {
 // thread per row: (A x)_i in CSR order, its distance to [lo_i, hi_i] and the row's
 // bound magnitude; the last block to finish reduces the per-block sums in a fixed
 // order, writes out[0] = ||r_p||_2 and out[1] = eps_p, and clears the counter.
-// ONE: a single block, which needs no counter (nor the memset before the launch) and is
-// bound by the latency of its loads.  VEC: cols and vals are 16-byte aligned; a thread then
-// reads its row in aligned groups of four, two groups in flight (200 rows: 12.7 us a call
-// among others, 10.7 so).  With many blocks the plain walk is the faster one (5M nonzeros
-// in rows of 25: 60 us against 64 in groups of four, and 83 to 88 with the matrix staged in
-// shared memory, whose barriers cost more than its coalesced loads save).
-template <bool ONE, bool VEC>
+// ONE: a single block, which needs no counter nor the memset before the launch (200 rows
+// of a set cover: 13.2 us a call among others, 10.2 so).  A row is walked entry by entry:
+// aligned groups of four with two in flight gained nothing there, took 31.0 us against 22.8
+// on 60 rows of 110 entries, 49.9 against 29.7 on 50 rows of 200 and 64 against 60 on 5M
+// nonzeros in rows of 25; the matrix staged in shared memory took 83 to 88 on the last (its
+// barriers cost more than its coalesced loads save).
+template <bool ONE>
 __global__ void __launch_bounds__(kNaThreads) k_primal_residual_noalloc(
     NoAllocScratch* sc, long long m, const long long* __restrict__ rowptr, const int* __restrict__ cols,
     const double* __restrict__ vals, const double* __restrict__ x, const double* __restrict__ lo,
@@ -62,51 +62,7 @@ __global__ void __launch_bounds__(kNaThreads) k_primal_residual_noalloc(
   if (i < m) {
     double ax = 0.0;
     const long long p0 = rowptr[i], p1 = rowptr[i + 1];
-    if (VEC) {
-      const long long nnz = rowptr[m];
-      auto group = [&](long long p, int (&c)[4], double (&v)[4]) {
-        if (p >= p1) {
-          c[0] = c[1] = c[2] = c[3] = -1;
-        } else if (p + 4 <= nnz) {
-          const int4 t = __ldg(reinterpret_cast<const int4*>(cols + p));
-          const double2 a = __ldg(reinterpret_cast<const double2*>(vals + p));
-          const double2 b = __ldg(reinterpret_cast<const double2*>(vals + p) + 1);
-          c[0] = t.x; c[1] = t.y; c[2] = t.z; c[3] = t.w;
-          v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-        } else {
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (p + e < p1) {
-              c[e] = __ldg(cols + p + e);
-              v[e] = __ldg(vals + p + e);
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (p + e < p0 || p + e >= p1) c[e] = -1;
-      };
-      for (long long p = p0 & ~3LL; p < p1; p += 8) {
-        int c[8], ca[4], cb[4];
-        double v[8], va[4], vb[4], g[8];
-        group(p, ca, va);
-        group(p + 4, cb, vb);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          c[e] = ca[e];
-          c[4 + e] = cb[e];
-          v[e] = va[e];
-          v[4 + e] = vb[e];
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          if (c[e] >= 0) g[e] = __ldg(x + c[e]);
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          if (c[e] >= 0) ax = fma(v[e], g[e], ax);
-      }
-    } else {
-      for (long long p = p0; p < p1; ++p) ax += vals[p] * x[cols[p]];
-    }
+    for (long long p = p0; p < p1; ++p) ax += vals[p] * x[cols[p]];
     const double l = lo[i], h = hi[i];
     const double proj = ax < l ? l : (ax > h ? h : ax);
     const double r = ax - proj;
@@ -220,7 +176,6 @@ extern "C" int scylla_primal_residual_noalloc(int64_t m, const int64_t* rowptr, 
   const int rc = scratch_for_current_device(&sc);
   if (rc != SCYLLA_OK) return rc;
   const int blocks = int((m + kNaThreads - 1) / kNaThreads);
-  const bool vec = (reinterpret_cast<uintptr_t>(cols) | reinterpret_cast<uintptr_t>(vals)) % 16 == 0;
   cudaError_t e = cudaSuccess;
   // every call of several blocks clears the arrival counter on its own stream before its
   // kernel: a finished kernel leaves it at zero, but one that failed part way (or a launch
@@ -231,9 +186,7 @@ extern "C" int scylla_primal_residual_noalloc(int64_t m, const int64_t* rowptr, 
                       cudaGetErrorString(e));
     return SCYLLA_ERR_CUDA;
   }
-  const auto k = blocks > 1 ? k_primal_residual_noalloc<false, false>
-                 : vec      ? k_primal_residual_noalloc<true, true>
-                            : k_primal_residual_noalloc<true, false>;
+  const auto k = blocks > 1 ? k_primal_residual_noalloc<false> : k_primal_residual_noalloc<true>;
   k<<<blocks, kNaThreads, 0, st>>>(sc, (long long)m, (const long long*)rowptr, cols, vals, x, row_lo, row_hi, out);
   e = cudaGetLastError();
   if (e != cudaSuccess) {
