@@ -257,19 +257,22 @@ struct NoPro {
   __device__ __forceinline__ bool operator()() const { return true; }
 };
 
-// entries that a lane gathers ahead of its sum where it gathers the entries it sums
-constexpr int kOwnAhead = 8;
+// entries that a lane gathers ahead of its sum where it gathers the entries it sums; in the
+// persistent kernel, whose attempts share the registers, fewer (640 attempts with a check
+// every 64, FP32-mixed, 8 / 4: packing/covering 50k x 100k 15.6 / 14.9 ms, 200k x 500k 52.0 /
+// 48.5; the checks out of line 15.8 and 56.1)
+constexpr int kOwnAhead = 8, kOwnAheadPersistent = 4;
 
 // Check form of the gather over FP32 iterates: every row sum is a chain of FP64 fused
 // multiply-adds of a value and an exactly converted entry, in CSR order (one FP64
 // instruction per nonzero and vector instead of a conversion, a product and a sum).
 // The multi-row path stages the tile's indices and values in shared memory, and the lane
-// that sums an entry gathers it, kOwnAhead entries at a time: the gathered entries need no
+// that sums an entry gathers it, AHEAD entries at a time: the gathered entries need no
 // way through shared memory, and neighbouring rows with neighbouring columns (network and
 // multi-period models) gather whole lines.  (packing/covering 200k x 500k: column check
 // 127 -> 99 us, row check 162 -> 141.)
 // smw holds kSmemPerWarp doubles, then kSmemPerWarp ints.
-template <int NV, typename Gather, typename Epi>
+template <int NV, int AHEAD, typename Gather, typename Epi>
 __device__ __forceinline__ void spmv_tiles_fma(const int2* __restrict__ tiles, int ntiles,
                                                const int* __restrict__ rowptr, const int* __restrict__ cols,
                                                const double* __restrict__ vals, Gather& gat, Epi& epi,
@@ -344,13 +347,13 @@ __device__ __forceinline__ void spmv_tiles_fma(const int2* __restrict__ tiles, i
 #pragma unroll
       for (int k = 0; k < NV; ++k) s[k] = 0.0;
       if (mine) {
-        for (int q = q0 + sub; q < q1; q += kOwnAhead * L) {
-          float g[kOwnAhead][NV];
+        for (int q = q0 + sub; q < q1; q += AHEAD * L) {
+          float g[AHEAD][NV];
 #pragma unroll
-          for (int u = 0; u < kOwnAhead; ++u)
+          for (int u = 0; u < AHEAD; ++u)
             if (q + u * L < q1) gat(sc[skew(q + u * L)], g[u]);
 #pragma unroll
-          for (int u = 0; u < kOwnAhead; ++u)
+          for (int u = 0; u < AHEAD; ++u)
             if (q + u * L < q1) {
               const double a = smw[skew(q + u * L)];
 #pragma unroll
@@ -1222,13 +1225,13 @@ __global__ void __launch_bounds__(kThreads, 3) k_dual_as(DevLP<float> d) {
 
 // the two-vector FP64 gather of a check: FP32 iterates take the fused form; FP64
 // iterates the product form (their gathered entries need no conversion)
-template <typename Gather, typename Epi>
+template <int AHEAD, typename Gather, typename Epi>
 __device__ __forceinline__ void check_gather(const int2* tiles, int ntiles, const int* rowptr, const int* cols,
                                              const double* vals, Gather& gat, Epi& epi, double* smw,
                                              const float* /*tag*/) {
-  spmv_tiles_fma<2>(tiles, ntiles, rowptr, cols, vals, gat, epi, smw);
+  spmv_tiles_fma<2, AHEAD>(tiles, ntiles, rowptr, cols, vals, gat, epi, smw);
 }
-template <typename Gather, typename Epi>
+template <int AHEAD, typename Gather, typename Epi>
 __device__ __forceinline__ void check_gather(const int2* tiles, int ntiles, const int* rowptr, const int* cols,
                                              const double* vals, Gather& gat, Epi& epi, double* smw,
                                              const double* /*tag*/) {
@@ -1339,8 +1342,9 @@ __device__ __forceinline__ void check_cols_phase(const DevLP<T>& d, const SlotVi
     g[0] = y;
     g[1] = av;
   };
-  check_gather(d.t_tiles, d.t_ntiles, d.t_rowptr, d.t_cols, d.t_vals64, gat, epi,
-               sm + (threadIdx.x >> 5) * 2 * kSmemPerWarp, static_cast<const T*>(nullptr));
+  constexpr int kAhead = Coh ? kOwnAheadPersistent : kOwnAhead;
+  check_gather<kAhead>(d.t_tiles, d.t_ntiles, d.t_rowptr, d.t_cols, d.t_vals64, gat, epi,
+                       sm + (threadIdx.x >> 5) * 2 * kSmemPerWarp, static_cast<const T*>(nullptr));
   block_store_partials<kNC1>(epi.acc, part);
   const unsigned long long h = warp_sum_u64(epi.h);
   if ((threadIdx.x & 31) == 0 && h != 0ULL) atomicAdd(hash, h);
@@ -1407,8 +1411,9 @@ __device__ __forceinline__ void check_rows_phase(const DevLP<T>& d, const SlotVi
     g[0] = gload<Coh>(xc + j);
     g[1] = gload<Coh>(xa + j);
   };
-  check_gather(d.a_tiles, d.a_ntiles, d.a_rowptr, d.a_cols, d.a_vals64, gat, epi,
-               sm + (threadIdx.x >> 5) * 2 * kSmemPerWarp, static_cast<const T*>(nullptr));
+  constexpr int kAhead = Coh ? kOwnAheadPersistent : kOwnAhead;
+  check_gather<kAhead>(d.a_tiles, d.a_ntiles, d.a_rowptr, d.a_cols, d.a_vals64, gat, epi,
+                       sm + (threadIdx.x >> 5) * 2 * kSmemPerWarp, static_cast<const T*>(nullptr));
   block_store_partials<kNC2>(epi.acc, part);
 }
 
