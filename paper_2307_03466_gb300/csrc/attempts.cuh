@@ -29,7 +29,6 @@
 #pragma once
 
 constexpr int kResTile = kTileNnz;  // entries of a tile's slot in shared memory
-constexpr int kResMaxPart = 512;    // tiles of a side in the cluster scope
 constexpr int kResMaxVb = 8;        // virtual blocks per block in the grid scope
 
 // most threads of a block: as many warps per SM as the launched form keeps resident
@@ -37,6 +36,13 @@ constexpr int kResMaxVb = 8;        // virtual blocks per block in the grid scop
 template <typename T>
 struct ResidentThreads {
   static constexpr int value = sizeof(T) == 4 ? 1024 : 512;
+};
+
+// most tiles of a side in the cluster scope: FP32 what 8 blocks of 32 warps hold beside three
+// control warps each; FP64 where the grid's SMs are worth more than its barrier (resident_plan)
+template <typename T>
+struct ResidentTiles {
+  static constexpr int value = sizeof(T) == 4 ? 8 * (ResidentThreads<T>::value / 32 - 3) : 64;
 };
 
 struct ResidentArgs {
@@ -283,7 +289,7 @@ __global__ void __launch_bounds__(ResidentThreads<T>::value, 1)
   __shared__ StepPre spre;
   __shared__ T red[kNP + kND];
   __shared__ T shw[2][kResMaxVb][8];
-  constexpr int kP = VS ? kResMaxPart : 1;
+  constexpr int kP = VS ? ResidentTiles<T>::value : 1;
   __shared__ T bpart[4 * kP];  // cluster scope: primal sums (two buffers), dual sums (pairs)
   if (d.ctl->done || d.ctl->k >= d.ctl->iter_limit) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5, P = gridDim.x;
@@ -496,7 +502,8 @@ __global__ void __launch_bounds__(ResidentThreads<T>::value, 1)
 template <typename T>
 static const void* resident_kernel(const ResidentPlan& p) {
   if (p.scope == kScopeCluster) return (const void*)k_attempts<T, kScopeCluster, 1>;
-  if (sizeof(T) == 8 && p.tpw == 2) return (const void*)k_attempts<T, kScopeGrid, 2>;
+  if constexpr (sizeof(T) == 8)
+    if (p.tpw == 2) return (const void*)k_attempts<T, kScopeGrid, 2>;
   return (const void*)k_attempts<T, kScopeGrid, 1>;
 }
 
@@ -565,7 +572,7 @@ bool resident_plan(const DevLP<T>& d, ResidentPlan* out) {
   // / 522 us, 330 tiles - / 610 / 562; FP64 (bound by the SMs' FP64 pipes), 44 tiles 659 /
   // 596 / 760, 125 tiles - / 834 / 774.
   const int top = sizeof(T) == 4 ? 8 : 16;
-  if (spread && most <= (sizeof(T) == 4 ? kResMaxPart : 64)) {
+  if (spread && most <= ResidentTiles<T>::value) {
     for (int P = most > 8 ? top : most > 2 ? 4 : 1; P >= 1; P /= 2) {
       const int per = (most + P - 1) / P;
       if (per + 3 > warps) break;
