@@ -571,6 +571,10 @@ bool resident_plan(const DevLP<T>& d, ResidentPlan* out) {
   // blocks.  Measured per 64 attempts, cluster of 8 / 16 / grid: FP32, 125 tiles 397 / 398
   // / 522 us, 330 tiles - / 610 / 562; FP64 (bound by the SMs' FP64 pipes), 44 tiles 659 /
   // 596 / 760, 125 tiles - / 834 / 774.
+  // Few tiles take fewer blocks; with their check, 1 / 4 / 8 / 16 blocks: FP64, 2 tiles 397 /
+  // 418 / 419 / 432 us, 8 tiles 557 / 425 / 427 / 439, 9 tiles 603 / 434 / 430 / 440, 24 tiles
+  // - / 526 / 451 / 460; FP32, 2 tiles 187 / 236 / 239 / 246, 8 tiles 201 / 239 / 240 / 248, 24
+  // tiles 286 / 249 / 246 / 262 (one block is the faster one there up to some 16 tiles).
   const int top = sizeof(T) == 4 ? 8 : 16;
   if (spread && most <= ResidentTiles<T>::value) {
     for (int P = most > 8 ? top : most > 2 ? 4 : 1; P >= 1; P /= 2) {
