@@ -34,11 +34,13 @@ __device__ __forceinline__ int row_lanes(int nr) {
   return 1 << (31 - __clz(l));
 }
 // Its base-2 logarithm by shifts: an integer division by a run-time value is some twenty
-// instructions, and two more divisions map a lane to its row.  (spmv_tiles and
-// spmv_tiles_async keep the divisions: their L = 1 tiles branch past them, and the shift
-// form was 3 to 7% slower on the multicommodity-flow workload; 128 attempts of 1000 nodes and
-// 500 commodities, both kernels in the asynchronous-copy form, 20.3 against 18.5 ms, with the
-// wide primal 14.6 against 14.2.)
+// instructions, and two more divisions map a lane to its row.  (spmv_tiles keeps the
+// divisions: its L = 1 tiles branch past them, and the shift form was 3 to 7% slower on the
+// multicommodity-flow workload.  Of the asynchronous-copy forms, which overlap their
+// successor's start, the pair of both is the faster with divisions in both, 128 attempts of
+// 12.8M nonzeros 18.5 ms, 20.3 with shifts and 21.3 with shifts in the dual alone; the dual
+// beside another primal with shifts, 640 attempts of 3.8M 23.8 ms against 24.3, 19.2M 97.8
+// against 99.4, 25.6M 128 against 130, though 12.8M 70.1 against 68.6.)
 __device__ __forceinline__ int row_lanes_log2(int nr) { return nr >= 32 ? 0 : nr > 1 ? __clz(nr - 1) - 27 : 5; }
 
 // The tiles of a warp: tile t goes to block t mod G and, within the block, to warp
@@ -511,7 +513,8 @@ struct AsyncStage {
   V pre[5][32];
 };
 
-template <typename V, typename Gather, typename Epi>
+// kDiv: the lane map by divisions (row_lanes_log2)
+template <bool kDiv, typename V, typename Gather, typename Epi>
 __device__ __forceinline__ void spmv_tiles_async(const int2* __restrict__ tiles, int ntiles,
                                                  const int* __restrict__ rowptr, const int* __restrict__ cols,
                                                  const V* __restrict__ vals, Gather& gat, Epi& epi,
@@ -568,8 +571,9 @@ __device__ __forceinline__ void spmv_tiles_async(const int2* __restrict__ tiles,
       long_row_sum<1, true>(p0, p1, cols, vals, gat, s);
       if (lane == 0) epi.finish(r0, s, pre);
     } else {
-      const int nr = r1 - r0, L = row_lanes(nr), sub = L > 1 ? lane % L : 0;
-      const int rl = L > 1 ? lane / L : lane;
+      const int nr = r1 - r0, sh = kDiv ? 0 : row_lanes_log2(nr), L = kDiv ? row_lanes(nr) : 1 << sh;
+      const int sub = kDiv ? (L > 1 ? lane % L : 0) : lane & (L - 1);
+      const int rl = kDiv ? (L > 1 ? lane / L : lane) : lane >> sh;
       int q0 = 0, q1 = 0;
       typename Epi::Pre pre{};
       if (rl < nr) {
@@ -1187,13 +1191,15 @@ __global__ void __launch_bounds__(kThreads, 3) k_primal_as(DevLP<float> d) {
     const float* __restrict__ yc = d.Y[v.cur];
     auto gat = [&](int i, float(&g)[1]) { g[0] = __ldg(yc + i); };
     const int w = threadIdx.x >> 5;
-    spmv_tiles_async<float>(d.t_tiles, d.t_ntiles, d.t_rowptr, d.t_cols, d.t_vals, gat, epi, sm + w * kSmemPerWarp,
+    spmv_tiles_async<true, float>(d.t_tiles, d.t_ntiles, d.t_rowptr, d.t_cols, d.t_vals, gat, epi, sm + w * kSmemPerWarp,
                             stg[w], v.do_avg ? 31 : 15);
   }
   const float acc[kNP] = {epi.acc};
   block_store_partials<kNP>(acc, acc_part<float>(d.part_p));
 }
 
+// kDiv: beside the asynchronous-copy primal (row_lanes_log2)
+template <bool kDiv>
 __global__ void __launch_bounds__(kThreads, 3) k_dual_as(DevLP<float> d) {
   typedef AccOf<float>::type A;
   Control* ctl = d.ctl;
@@ -1207,7 +1213,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_dual_as(DevLP<float> d) {
   const float* __restrict__ xn = d.X[v.nxt];
   auto gat = [&](int j, float(&g)[1]) { g[0] = __ldg(xn + j); };
   const int w = threadIdx.x >> 5;
-  spmv_tiles_async<float>(d.a_tiles, d.a_ntiles, d.a_rowptr, d.a_cols, d.a_vals, gat, epi, sm + w * kSmemPerWarp,
+  spmv_tiles_async<kDiv, float>(d.a_tiles, d.a_ntiles, d.a_rowptr, d.a_cols, d.a_vals, gat, epi, sm + w * kSmemPerWarp,
                           stg[w], v.do_avg ? 31 : 15);
   const A acc[kND] = {epi.acc0, epi.acc1};
   block_store_partials<kND>(acc, acc_part<float>(d.part_d));
@@ -3078,7 +3084,8 @@ cudaError_t launch_dual(const DevLP<T>& d, cudaStream_t st) {
   switch (d.form_d) {
     case kFormStaged: return launch_step_kernel<T>(k_dual_st<T>, d.grid_d, d, st, Staged<T>::kBlockBytes);
     case kFormAsync:
-      if constexpr (std::is_same<T, float>::value) return launch_step_kernel<float>(k_dual_as, d.grid_d, d, st);
+      if constexpr (std::is_same<T, float>::value)
+        return launch_step_kernel<float>(d.form_p == kFormAsync ? k_dual_as<true> : k_dual_as<false>, d.grid_d, d, st);
       return cudaErrorInvalidValue;
     case kFormPrefetch: return launch_step_kernel<T>(k_dual<T, kFormPrefetch>, d.grid_d, d, st);
     case kFormWide: return launch_step_kernel<T>(k_dual<T, kFormWide>, d.grid_d, d, st);
@@ -3171,7 +3178,7 @@ int occupancy_grid(int side, int form, int work_tiles) {
     k = side == 0 ? k_primal_st<T> : k_dual_st<T>;
     smem = Staged<T>::kBlockBytes;
   } else if (form == kFormAsync) {
-    if constexpr (std::is_same<T, float>::value) k = side == 0 ? k_primal_as : k_dual_as;
+    if constexpr (std::is_same<T, float>::value) k = side == 0 ? k_primal_as : k_dual_as<false>;
     else k = side == 0 ? k_primal<T, kFormPlain> : k_dual<T, kFormPlain>;
   } else if (form == kFormWide) k = side == 0 ? k_primal<T, kFormWide> : k_dual<T, kFormWide>;
   else if (form == kFormPrefetch) k = side == 0 ? k_primal<T, kFormPrefetch> : k_dual<T, kFormPrefetch>;
