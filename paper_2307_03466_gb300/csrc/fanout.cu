@@ -451,16 +451,18 @@ __device__ __forceinline__ void fan_block_sums(A (&acc)[NSUM][FanGeo<VEC, CHUNK>
   }
 }
 
-// Whether an attempt's dual step, or a check's row half, has an objective to work on.
-// The kernel after it (and the copies after that one) takes the answer from the state:
-// the control kernels count finished objectives themselves, so a block of theirs that
-// looked at the count could find it changed by its own launch and skip its duties (the
-// attempt's count, an earlier flag's reset).
+// Whether every objective is finished, for an attempt's dual step and a check's row half,
+// which then note it in the state (k_finit clears the note): the control kernel after them,
+// and the copies after that one, go by the note.  The control kernels count finished
+// objectives themselves, so a block of theirs that looked at the count could find it
+// changed by its own launch and skip its duties (the attempt's count, an earlier flag's
+// reset).  A kernel with work to do writes nothing: a store ahead of the row half's loop
+// took six registers more and 2.7% of its time, one at the dual's end 6%.
 template <typename T>
-__device__ __forceinline__ bool fan_live(const DevFan<T>& F) {
-  const bool live = *F.n_done < F.K;
-  if (blockIdx.x == 0 && threadIdx.x == 0) F.state->live = live ? 1 : 0;
-  return live;
+__device__ __forceinline__ bool fan_over(const DevFan<T>& F) {
+  if (*F.n_done < F.K) return false;
+  if (blockIdx.x == 0 && threadIdx.x == 0) F.state->over = 1;
+  return true;
 }
 
 // Primal SpMM of one attempt for every objective (Algorithm 1, primal step):
@@ -601,7 +603,7 @@ template <typename T, int VEC, int CHUNK>
 __global__ void __launch_bounds__(kFThreads, sizeof(T) == 4 && !(VEC == 4 && CHUNK == 32) ? 4 : 3) k_fdual(DevFan<T> F) {
   typedef typename AccOf<T>::type A;
   typedef FanGeo<VEC, CHUNK> G;
-  if (!fan_live(F)) return;
+  if (fan_over(F)) return;
   __shared__ double sh[kFWarps * 2 * kFK];
   __shared__ __align__(16) FanShared<T> S;
   __shared__ __align__(16) FanStage<T, VEC> E;
@@ -769,7 +771,7 @@ constexpr int kFStepThreads = 3 * 32;
 template <typename T>
 __global__ void __launch_bounds__(kFStepThreads) k_fstep_control(DevFan<T> F) {
   FanState* st = F.state;
-  if (!st->live) return;  // nothing attempted: the pools keep their roles
+  if (st->over) return;  // nothing attempted: the pools keep their roles
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ++*F.kglob;
     ++st->att;
@@ -916,7 +918,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_fcheck_cols(DevFan<T> F) {
 // Row half of a check, laid out as the column half.
 template <typename T>
 __global__ void __launch_bounds__(kFThreads, 3) k_fcheck_rows(DevFan<T> F) {
-  if (!fan_live(F)) return;
+  if (fan_over(F)) return;
   __shared__ double sh[kFWarps * kNC2 * 32];
   const int lane = threadIdx.x & 31, halves = fan_halves(F.K);
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
@@ -981,7 +983,7 @@ constexpr int kFCheckThreads = (kNC1 + kNC2) * 32;
 template <typename T>
 __global__ void __launch_bounds__(kFCheckThreads) k_fcheck_control(DevFan<T> F) {
   FanState* st = F.state;
-  if (!st->live) return;
+  if (st->over) return;
   const long long k0 = *F.kglob;
   constexpr bool f32 = sizeof(T) == 4;
   const int k = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1051,7 +1053,7 @@ __global__ void __launch_bounds__(kFCheckThreads) k_fcheck_control(DevFan<T> F) 
 template <typename T, bool RST>
 __global__ void __launch_bounds__(kFThreads) k_fcopy(DevFan<T> F) {
   const FanState* st = F.state;
-  if (!st->live) return;  // no attempt or check was made: the flags are an earlier one's
+  if (st->over) return;  // no attempt or check was made: the flags are an earlier one's
   const unsigned char* flag = RST ? st->rst : st->rej;
   // the flagged objectives, ascending
   __shared__ int list[kFK];
@@ -1123,6 +1125,7 @@ __global__ void k_finit(DevFan<T> F, double tol, long long iter_limit, int stall
   if (k == 0) {
     *F.kglob = 0;
     *F.n_done = 0;
+    F.state->over = 0;
   }
   if (k >= F.K) return;
   Control* c = &F.ctl[k];

@@ -199,7 +199,7 @@ struct FanState {
   unsigned long long att;     // attempts since seeding: X[att & 1], Y[.], AX[.] hold the current points
   unsigned char rej[64];      // 1: rejected in the last attempt (next pool -> current), written every attempt
   unsigned char rst[64];      // 1: restarted to or finished with the average (average -> current), every check
-  int live;                   // the attempt or check under way has an objective that is not finished
+  int over;                   // every objective was finished before the attempt or check under way
 };
 
 // K objectives of one LP solved together: K-wide vectors are row-major with 64

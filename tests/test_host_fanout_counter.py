@@ -25,4 +25,4 @@ def test_kernels_that_count_finished_objectives_do_not_read_the_count():
     writers = [k for k, b in bodies.items() if re.search(r"atomicAdd\(F\.n_done", b)]
     assert sorted(writers) == ["k_fcheck_control", "k_fstep_control"]
     for k in writers:
-        assert not re.search(r"\*F\.n_done\b|fan_live\(", bodies[k]), k
+        assert not re.search(r"\*F\.n_done\b|fan_over\(", bodies[k]), k
