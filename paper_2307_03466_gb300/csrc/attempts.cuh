@@ -459,9 +459,7 @@ __global__ void __launch_bounds__(ResidentThreads<T>::value, 1)
         if (Rt[i].t >= 0) sp[i] = res_rowsum<T, VS>(St, Rt[i], idx_t, val_t, VS ? ys : d.Y[v.nxt], sm);
     }
     __syncthreads();
-    // accepted (a non-finite sum ends the solve and leaves aty_valid as the attempt
-    // before set it: the failed candidate must not replace that attempt's point)
-    if (!sc.aty_valid && !sc.done) {
+    if (!sc.aty_valid) {  // accepted
 #pragma unroll
       for (int i = 0; i < TPW; ++i) {
         xc[i] = xn[i];

@@ -563,6 +563,7 @@ __device__ void step_control<double>(Control* c, const StepPre& p, double dx2, d
   if (!isfinite(dx2) || !isfinite(dy2) || !isfinite(inter)) {
     c->done = 1;
     c->status = SCYLLA_NUMERICAL;
+    c->aty_valid = 1;  // not accepted: the point stays, and its A^T y (k_attempts goes by this)
     return;
   }
   bool accept = true;
@@ -614,6 +615,7 @@ __device__ void step_control<float>(Control* c, const StepPre& p, float dx2, flo
   if (!isfinite(dx2) || !isfinite(dy2) || !isfinite(inter)) {
     c->done = 1;
     c->status = SCYLLA_NUMERICAL;
+    c->aty_valid = 1;  // as above
     sync_step_state(c);
     return;
   }
